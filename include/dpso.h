@@ -103,11 +103,11 @@ typedef struct dpso_stats {
     int64_t two_opt_runs;   /* generations in which the edge exchange ran */
     int32_t device_status;  /* sticky device-side error code (DPSO_OK if none) */
     int32_t reserved;
-    int64_t two_opt_evaluated; /* candidate pairs the kernels evaluated: at most
-                                  two_opt_pairs, fewer when a pass reuses the
-                                  previous pass's row minima (rows a move left
-                                  unchanged are not evaluated again); a count
-                                  of this process's work, not saved in a state */
+    int64_t two_opt_evaluated; /* candidate pairs the kernels evaluated, counted up
+                                  to two_opt_pairs: fewer when a pass knows from
+                                  earlier ones that a pair cannot be the best; a
+                                  count of this process's work, not saved in a
+                                  state */
 } dpso_stats;
 
 /* Per-phase device time of a swarm's generations while timing is on
@@ -174,11 +174,8 @@ int dpso_two_opt(const int32_t *C_dev, int32_t n, uint16_t *tours_dev, int32_t c
 /*
  * dpso_two_opt without any device allocation (the paper has no counterpart;
  * this is a deployment variant).  Same arguments, the same tours, costs,
- * pair and move counts, and the same synchronisation as dpso_two_opt, but it
- * always runs the general (untiled) 2-opt kernel, which is slower for tours
- * the tiled kernel takes (n <= 4145): the tiled kernel reads four row-shifted
- * copies of the cost matrix that would have to be allocated.  Its scratch --
- * error word, work queue, totals, the task descriptor and per-tour pass /
+ * pair and move counts, and the same synchronisation as dpso_two_opt, and it
+ * runs the same kernel.  Its scratch -- error word, work queue, totals, the task descriptor and per-tour pass /
  * move counts -- lives in one fixed 128 KiB device array inside the library
  * (held by every GPU that loads it, until exit) instead of being allocated
  * per call; it calls no allocating routine.
@@ -344,32 +341,36 @@ int dpso_batch_step(dpso_batch *b, int32_t iterations, void *stream);
 /* Launch shape of the tiled 2-opt kernel: tile height (rows: 32 / 30 / 24 /
  * 16 / 8), tours per CTA (1 / 2 / 4) and tiles of one tour in flight at once
  * (1, or 2 with one tour per CTA: two 8-warp subgroups of a 16-warp CTA).
- * All zero means the defaults for the longest tour of the batch. */
+ * All zero means the list kernel, which every exchange runs on unless a shape
+ * is pinned here. */
 typedef struct {
     int32_t rows;
     int32_t tours_per_cta;
     int32_t tiles_in_flight;
 } dpso_two_opt_shape;
 
-/* Picks the 2-opt launch shape for this batch by timing every shape that fits
- * on scratch copies of the members' current tours (at most 8 moves per tour
- * each, so the probe costs a few passes; best called right after creation).
- * Results do not depend on the choice.  *chosen (may be NULL) receives the
- * shape in use.  Synchronises `stream`. */
+/* Picks the 2-opt kernel and launch shape for this batch by timing the list
+ * kernel and every tiled shape that fits on scratch copies of the members'
+ * current tours (at most 32 moves per tour each; best called right after
+ * creation).  Results do not depend on the choice.  *chosen (may be NULL)
+ * receives the tiled shape in use, or where the list kernel was faster the
+ * tiled kernel's default shape (dpso_two_opt_default_shape).  Synchronises
+ * `stream`. */
 int dpso_batch_autotune(dpso_batch *b, dpso_two_opt_shape *chosen, void *stream);
-/* Sets the 2-opt launch shape by hand (NULL or all zero: the defaults).
- * DPSO_ERR_ARG when the shape is not one of the above, does not fit in shared
- * memory for the longest member, or the members lack the row-shifted cost
- * copies the tiled kernel reads.  Results do not depend on the shape.
+/* Sets the 2-opt launch shape by hand (NULL or all zero: the list kernel).
+ * DPSO_ERR_ARG when the shape is not one of the above or does not fit in
+ * shared memory for the longest member; DPSO_ERR_NO_MEMORY without room for
+ * the row-shifted cost copies the tiled kernel reads (made at the first
+ * pinned shape).  Results do not depend on the shape.
  * Synchronises the batch's stream. */
 int dpso_batch_set_two_opt_shape(dpso_batch *b, const dpso_two_opt_shape *shape);
-/* The 2-opt launch shape used when none is pinned, for a launch over `count`
- * tours of n viewpoints on a GPU with `num_sms` SMs (a launch implementation
- * choice; the paper has none).  Up to n = 256: 32-row tiles, two tours per
+/* The tiled 2-opt kernel's default launch shape for a launch over `count` tours
+ * of n viewpoints on a GPU with `num_sms` SMs (a launch implementation choice;
+ * the paper has none; unpinned launches run the list kernel instead).  Up to n = 256: 32-row tiles, two tours per
  * CTA; beyond: the shape with the most tile rows in flight per SM, except that
  * tours whose tallest fitting tile has 16 rows or fewer take 8-row tiles with
  * two tours per CTA when those fit and count >= 2 * num_sms.  All zero when
- * no tiled shape fits (the general kernel runs).  Host only, no device call.
+ * no tiled shape fits.  Host only, no device call.
  * DPSO_ERR_ARG for a NULL out, n < 3, count < 0 or num_sms < 1. */
 int dpso_two_opt_default_shape(int32_t n, int32_t count, int32_t num_sms,
                                dpso_two_opt_shape *out);

@@ -27,7 +27,8 @@ COMMON = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
 SOURCES = {
     "cost.cu": ["-fmad=false"],
     "swarm.cu": [],
-    "two_opt.cu": [],
+    "two_opt_list.cu": [],
+    "two_opt_small.cu": [],
     "two_opt_tiled.cu": [],
     "node_swap_tiled.cu": [],
     "runtime.cu": [],

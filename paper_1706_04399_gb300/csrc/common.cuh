@@ -167,7 +167,7 @@ cudaError_t launch_gbest(const BatchView& b, int second, cudaStream_t st);
 cudaError_t launch_philox_draws(unsigned long long seed, uint32_t phase, uint32_t iter,
                                 uint32_t particle, int count, uint32_t* out, cudaStream_t st);
 
-// ---- launchers (two_opt.cu, two_opt_tiled.cu) ----
+// ---- launchers (two_opt_list.cu, two_opt_tiled.cu) ----
 // One 2-opt problem: best-improvement 2-opt on `count` tours of length n (row
 // stride ldt), updating tours, costs and (when pbest != nullptr) the pbest
 // arrays.  When `gate` is non-null nothing happens unless *gate != 0.
@@ -209,14 +209,23 @@ struct TwoOptBatch {
     const int* off;
     int nprob, total;
     int max_n;        // sizes shared memory and the tile height
-    bool shifted;     // every task has Cs: the tiled kernel may be used
-    int rows;         // tile height of the tiled kernel (0: the default for max_n)
+    bool shifted;     // every task has Cs: the tiled kernels may be used
+    int rows;         // tile height of the tiled 2-opt kernel (0: the list kernel)
     unsigned int* queue;
     int tpc;          // tours per CTA of the tiled kernel (0: the default for max_n)
     int tg;           // tile subgroups per tour of the tiled kernel (0: the default)
     int kind;         // exchange of every task: 0 edge exchange (2-opt), 1 node swap
 };
+// The exchange of b.kind: the node-swap kernel; the 2-opt on the list kernel
+// (short tours: two_opt_small.cu), or on the tiled kernel when a shape of it
+// is pinned (rows > 0).
 cudaError_t launch_two_opt(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+// ---- two_opt_small.cu: short tours ----
+int two_opt_small_threads(int n);  // threads per tour, 0 when n is too long
+cudaError_t launch_two_opt_small(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+// The launch configuration for many tours of up to n viewpoints, and the tours
+// one SM then holds: members that agree share a launch.
+int two_opt_class(int n, int* ctas);
 
 // ---- two_opt_tiled.cu: pipelined tiled variant (needs the shifted copies) ----
 // Row pitch (words) of the shifted copies and of the staged rows: room for a
@@ -256,7 +265,11 @@ bool two_opt_tiled_fits(int n, int rows, int tpc, int tg);  // a valid shape tha
 cudaError_t build_shifted_copies(const int* C, int ldc, int n, int* Cs, cudaStream_t st);
 cudaError_t launch_two_opt_tiled(const TwoOptBatch& b, int rows, int tpc, int tg, int num_sms,
                                  cudaStream_t st);
-cudaError_t launch_two_opt_general(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+// ---- two_opt_list.cu: the default 2-opt kernel, any n ----
+cudaError_t launch_two_opt_list(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+// Launch configuration (a number from 0) for tours of up to n viewpoints, and
+// the tours one SM then holds.
+int two_opt_list_class(int n, int* ctas);
 
 // ---- node_swap_tiled.cu: node-swap exchange (needs the shifted copies and
 // entries of C at most DPSO_NODE_SWAP_COST_MAX) ----
@@ -266,7 +279,6 @@ cudaError_t launch_node_swap_tiled(const TwoOptBatch& b, int num_sms, cudaStream
 
 // ---- runtime.cu ----
 __global__ void tours_valid_kernel(const uint16_t* tours, int n, int* err);
-int two_opt_rows(int n);
 int validate_params(const dpso_params* p);
 
 }  // namespace dpso

@@ -86,7 +86,7 @@ struct dpso_swarm {
     Consts k{};
     SwarmDev d{};
     int* C = nullptr;
-    int* Cs = nullptr;  // row-shifted copies of C for the TMA 2-opt (or null)
+    int* Cs = nullptr;  // row-shifted copies of C for the tiled exchange kernels (or null)
     uint16_t *X = nullptr, *V = nullptr, *P = nullptr, *G = nullptr;
     long long *F = nullptr, *PF = nullptr;
     unsigned long long* hash = nullptr;
@@ -315,6 +315,21 @@ int ensure_history(dpso_swarm* s, int need) {
     return DPSO_OK;
 }
 
+// The row-shifted copies of C that the tiled exchange kernels read: the node
+// swap's from the start, the 2-opt's when a batch pins a tiled shape.
+int ensure_shifted(dpso_swarm* s) {
+    if (s->Cs) return DPSO_OK;
+    const int n = s->k.n;
+    const int st = dalloc(&s->Cs, static_cast<size_t>(4) * n * shifted_ld(n), s->last);
+    if (st) return st;
+    if (build_shifted_copies(s->C, s->k.ldc, n, s->Cs, s->last) != cudaSuccess) {
+        cudaFree(s->Cs);
+        s->Cs = nullptr;
+        return DPSO_ERR_CUDA;
+    }
+    return DPSO_OK;
+}
+
 int read_ctl(dpso_swarm* s, Ctl* c) {
     CK(cudaStreamSynchronize(s->last));
     CK(cudaMemcpy(c, s->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
@@ -433,12 +448,12 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     int* Cs = nullptr;
-    if (e == cudaSuccess && herr == 0 && two_opt_tiled_rows(n) > 0) {
+    if (e == cudaSuccess && herr == 0 && kind == 1) {  // the node swap's row-shifted copies
         if (cudaMallocAsync(&Cs, sizeof(int) * 4 * static_cast<size_t>(n) * shifted_ld(n), st) !=
             cudaSuccess) {
             cudaGetLastError();
-            Cs = nullptr;  // 2-opt falls back to the kernel that stages rows itself
-            if (kind == 1) e = cudaErrorMemoryAllocation;
+            Cs = nullptr;
+            e = cudaErrorMemoryAllocation;
         } else {
             e = build_shifted_copies(C_dev, n, n, Cs, st);
         }
@@ -546,7 +561,6 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
     if (cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, s->device) !=
         cudaSuccess)
         return fail(DPSO_ERR_CUDA);
-    if (two_opt_rows(n) == 0) return fail(DPSO_ERR_RANGE);
     const bool node_swap = (p->flags & DPSO_FLAG_TWO_OPT) && (p->flags & DPSO_FLAG_NODE_SWAP);
     if (node_swap && node_swap_tiled_rows(n) == 0) return fail(DPSO_ERR_RANGE);
 
@@ -622,12 +636,7 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
         return fail2(DPSO_ERR_CUDA);
     if (herr & 1) return fail2(DPSO_ERR_ARG);
     if (herr & 2) return fail2(DPSO_ERR_RANGE);
-    if ((p->flags & DPSO_FLAG_TWO_OPT) && two_opt_tiled_rows(n) > 0) {
-        if ((st = dalloc(&s->Cs, static_cast<size_t>(4) * n * shifted_ld(n), ust)))
-            return fail2(st);
-        if (build_shifted_copies(s->C, k.ldc, n, s->Cs, ust) != cudaSuccess)
-            return fail2(DPSO_ERR_CUDA);
-    }
+    if (node_swap && (st = ensure_shifted(s))) return fail2(st);
     {
         SwarmMeta m{};
         m.desc.k = k;
@@ -872,8 +881,8 @@ struct dpso_batch {
     int* off = nullptr;         // device, ninst + 1
     BatchView bv{};
     bool any_two_opt = false;
-    bool shifted = true;                 // every exchanging member has the shifted copies
     std::vector<TwoOptTask> tasks;       // host: every exchanging member, by descending n
+    std::vector<dpso_swarm*> owners;     // the members the tasks belong to
     std::vector<TwoOptClass> cls;
     std::vector<cudaStream_t> side;      // capture streams of the classes after the first
     std::vector<cudaEvent_t> ev;         // fork, then one join per side stream
@@ -906,28 +915,35 @@ void free_batch(dpso_batch* b) {
     delete b;
 }
 
-// Default launch shape of the tiled kernel for tours of n viewpoints and the
-// resident CTAs per SM it gets (all zero: the general kernel).
+// Members whose tours run in one 2-opt launch: the same exchange and the same
+// launch configuration (a launch's shared memory follows its longest tour, so
+// short tours would run with too few tours per SM beside long ones).
 struct ShapeKey {
-    int kind = 0, rows = 0, tpc = 0, tg = 0, ctas = 0;
+    int kind = 0, cfg = 0, ctas = 0;
     bool operator==(const ShapeKey& o) const {
-        return kind == o.kind && rows == o.rows && tpc == o.tpc && tg == o.tg && ctas == o.ctas;
+        return kind == o.kind && cfg == o.cfg && ctas == o.ctas;
     }
 };
 
-ShapeKey default_shape(int n, bool shifted, int kind) {
+ShapeKey default_shape(int n, int kind) {
     ShapeKey k;
     k.kind = kind;
-    if (kind == 1) {  // node swap: one kernel shape per tile height
-        k.rows = node_swap_tiled_rows(n);
-        return k;
-    }
-    if (!shifted || two_opt_tiled_rows(n) == 0) return k;
-    k.rows = two_opt_tiled_rows(n);
-    k.tpc = two_opt_tiled_tpc(n, k.rows);
-    k.tg = two_opt_tiled_tg(n, k.rows, k.tpc);
-    k.ctas = two_opt_tiled_ctas(n, k.rows, k.tpc, k.tg);
+    if (kind == 1) k.cfg = node_swap_tiled_rows(n);  // one kernel shape per tile height
+    else k.cfg = two_opt_class(n, &k.ctas);
     return k;
+}
+
+// Gives every 2-opt member the row-shifted copies the tiled kernel reads.
+int ensure_batch_shifted(dpso_batch* b) {
+    for (size_t i = 0; i < b->tasks.size(); ++i) {
+        if (b->tasks[i].kind != 0) continue;
+        dpso_swarm* s = b->owners[i];
+        const int st = ensure_shifted(s);
+        if (st) return st;
+        CK(cudaStreamSynchronize(s->last));  // the batch's launches may be on another stream
+        b->tasks[i].Cs = s->Cs;
+    }
+    return DPSO_OK;
 }
 
 // Splits the exchanging members into launch classes: runs of members (by
@@ -943,7 +959,7 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
         if (pinned)
             k.kind = b->tasks[i].kind;  // one class per exchange kind
         else
-            k = default_shape(b->tasks[i].n, b->tasks[i].Cs != nullptr, b->tasks[i].kind);
+            k = default_shape(b->tasks[i].n, b->tasks[i].kind);
         if (i == 0 || !(k == keys.back())) {
             runs.push_back({i, i + 1});
             keys.push_back(k);
@@ -983,10 +999,6 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
             tb.rows = pinned->rows;
             tb.tpc = pinned->tours_per_cta;
             tb.tg = pinned->tiles_in_flight;
-        } else if (keys[c].rows > 0) {
-            tb.rows = keys[c].rows;
-            tb.tpc = keys[c].tpc;
-            tb.tg = keys[c].tg;
         }
     }
     // one capture stream and one join event per class after the first
@@ -1048,10 +1060,11 @@ int capture_batch(dpso_batch* b) {
     return e3 == cudaSuccess ? DPSO_OK : DPSO_ERR_CUDA;
 }
 
-// Times every shape that fits a class on scratch copies of its tours (gates
-// ignored, at most kProbeMoves moves per tour) and keeps the fastest.
+// Times the list kernel and every tiled shape that fits a class on scratch
+// copies of its tours (gates ignored, at most kProbeMoves moves per tour) and
+// keeps the fastest.
 int autotune_class(dpso_batch* b, dpso_batch::TwoOptClass& cl, cudaStream_t st) {
-    constexpr int kProbeMoves = 8;
+    constexpr int kProbeMoves = 32;
     if (cl.tb.kind != 0 || cl.tb.nprob <= 0 || !cl.tb.shifted ||
         two_opt_tiled_rows(cl.tb.max_n) == 0)
         return DPSO_OK;
@@ -1102,10 +1115,11 @@ int autotune_class(dpso_batch* b, dpso_batch::TwoOptClass& cl, cudaStream_t st) 
     float best = 1e30f;
     int rows_b = 0, tpc_b = 0, tg_b = 0;
     constexpr int kShapes[4][2] = {{1, 1}, {2, 1}, {4, 1}, {1, 2}};  // (tours per CTA, tiles)
-    for (int rows : {32, 30, 24, 16, 8}) {
+    for (int rows : {0, 32, 30, 24, 16, 8}) {  // 0: the list kernel
         for (const auto& sh : kShapes) {
             const int tpc = sh[0], tg = sh[1];
-            if (!two_opt_tiled_fits(cl.tb.max_n, rows, tpc, tg)) continue;
+            if (rows == 0 ? tpc != 1 || tg != 1 : !two_opt_tiled_fits(cl.tb.max_n, rows, tpc, tg))
+                continue;
             for (size_t i = 0; i < tasks.size(); ++i) {  // restore the tours
                 if (cudaMemcpy2DAsync(tasks[i].tours, sizeof(uint16_t) * tasks[i].ldt,
                                       orig[i].tours, sizeof(uint16_t) * orig[i].ldt,
@@ -1121,7 +1135,10 @@ int autotune_class(dpso_batch* b, dpso_batch::TwoOptClass& cl, cudaStream_t st) 
             if (cudaMemsetAsync(tb.queue, 0, sizeof(unsigned int), st) != cudaSuccess ||
                 cudaEventRecord(e0, st) != cudaSuccess)
                 return cleanup(DPSO_ERR_CUDA);
-            const cudaError_t le = launch_two_opt_tiled(tb, rows, tpc, tg, b->num_sms, st);
+            tb.rows = rows;
+            tb.tpc = tpc;
+            tb.tg = tg;
+            const cudaError_t le = launch_two_opt(tb, b->num_sms, st);
             if (le == cudaErrorInvalidValue || le == cudaErrorInvalidConfiguration) {
                 cudaGetLastError();  // this shape does not fit: skip it
                 continue;
@@ -1191,7 +1208,7 @@ int dpso_batch_create(dpso_batch** out, dpso_swarm* const* swarms, int32_t count
     for (int i : order) {
         if (!(swarms[i]->k.flags & DPSO_FLAG_TWO_OPT)) continue;
         b->tasks.push_back(swarm_task(swarms[i]));
-        b->shifted = b->shifted && swarms[i]->Cs != nullptr;
+        b->owners.push_back(swarms[i]);
     }
     b->any_two_opt = !b->tasks.empty();
     int st = DPSO_OK;
@@ -1240,6 +1257,12 @@ int dpso_batch_autotune(dpso_batch* b, dpso_two_opt_shape* chosen, void* stream)
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     CK(cudaStreamSynchronize(b->last));
     b->last = st;
+    // (without room for the copies only the list kernel can run: nothing to choose)
+    const int r0 = ensure_batch_shifted(b);
+    if (r0 && r0 != DPSO_ERR_NO_MEMORY) return r0;
+    // the classes are built again with the copies; a shape pinned before is timed anew
+    const int r1 = build_classes(b, nullptr);
+    if (r1) return r1;
     for (auto& cl : b->cls) {
         const int r = autotune_class(b, cl, st);
         if (r) return r;
@@ -1285,11 +1308,15 @@ int dpso_batch_set_two_opt_shape(dpso_batch* b, const dpso_two_opt_shape* shape)
         int max_n = 0;  // the shape applies to the edge-exchange (2-opt) members
         for (const TwoOptTask& t : b->tasks)
             if (t.kind == 0) max_n = std::max(max_n, t.n);
-        if (!b->shifted || max_n == 0 ||
+        if (max_n == 0 ||
             !two_opt_tiled_fits(max_n, shape->rows, shape->tours_per_cta, shape->tiles_in_flight))
             return DPSO_ERR_ARG;
     }
     CK(cudaStreamSynchronize(b->last));
+    if (!defaults) {
+        const int st = ensure_batch_shifted(b);
+        if (st) return st;
+    }
     const int st = build_classes(b, defaults ? nullptr : shape);
     if (st) return st;
     return capture_batch(b);

@@ -1,8 +1,7 @@
 // dpso_two_opt_noalloc: the standalone 2-opt entry point without any device
 // allocation.  Its scratch (error word, work queue, totals and per-tour pass /
-// move counts) lives in one fixed array inside the library.  It runs the
-// general (untiled) 2-opt kernel: the tiled kernel stages rows from four
-// row-shifted copies of the cost matrix, which would need an allocation.
+// move counts) lives in one fixed array inside the library.  It runs the list
+// kernel of dpso_two_opt, which reads the caller's cost matrix as it is.
 //
 // Who needs it: callers that must not allocate device memory while they run,
 // e.g. an on-board re-planning loop whose GPU memory is reserved once at

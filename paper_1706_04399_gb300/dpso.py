@@ -304,8 +304,8 @@ def dpso_probe_l2_read_gbs(nbytes: int = 24 << 20, reps: int = 40, stream=None) 
 
 
 def dpso_two_opt_default_shape(n: int, count: int, num_sms: int) -> tuple[int, int, int]:
-    """(tile rows, tours per CTA, tiles in flight) a launch over `count` tours
-    of n viewpoints takes when no shape is pinned; (0, 0, 0): the general kernel."""
+    """The tiled kernel's default (tile rows, tours per CTA, tiles in flight) for a
+    launch over `count` tours of n viewpoints; (0, 0, 0): no shape fits."""
     sh = dpso_two_opt_shape()
     _check(lib().dpso_two_opt_default_shape(n, count, num_sms, ctypes.byref(sh)),
            "dpso_two_opt_default_shape")
