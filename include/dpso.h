@@ -107,7 +107,7 @@ typedef struct dpso_stats {
                                   to two_opt_pairs: fewer when a pass knows from
                                   earlier ones that a pair cannot be the best; a
                                   count of this process's work, not saved in a
-                                  state */
+                                  state.  The node swap reports two_opt_pairs. */
 } dpso_stats;
 
 /* Per-phase device time of a swarm's generations while timing is on

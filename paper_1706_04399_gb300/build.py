@@ -30,7 +30,7 @@ SOURCES = {
     "two_opt_list.cu": [],
     "two_opt_small.cu": [],
     "two_opt_tiled.cu": [],
-    "node_swap_tiled.cu": [],
+    "node_swap.cu": [],
     "runtime.cu": [],
     "two_opt_noalloc.cu": [],
     "probe.cu": [],

@@ -271,11 +271,11 @@ cudaError_t launch_two_opt_list(const TwoOptBatch& b, int num_sms, cudaStream_t 
 // the tours one SM then holds.
 int two_opt_list_class(int n, int* ctas);
 
-// ---- node_swap_tiled.cu: node-swap exchange (needs the shifted copies and
-// entries of C at most DPSO_NODE_SWAP_COST_MAX) ----
-size_t node_swap_tiled_smem(int n, int rows);
-int node_swap_tiled_rows(int n);  // 0 when no tile height fits
-cudaError_t launch_node_swap_tiled(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+// ---- node_swap.cu: node-swap exchange (entries of C at most
+// DPSO_NODE_SWAP_COST_MAX) ----
+bool node_swap_fits(int n);
+int node_swap_class(int n);  // launch configuration: members that agree share a launch
+cudaError_t launch_node_swap(const TwoOptBatch& b, int num_sms, cudaStream_t st);
 
 // ---- runtime.cu ----
 __global__ void tours_valid_kernel(const uint16_t* tours, int n, int* err);

@@ -86,7 +86,7 @@ struct dpso_swarm {
     Consts k{};
     SwarmDev d{};
     int* C = nullptr;
-    int* Cs = nullptr;  // row-shifted copies of C for the tiled exchange kernels (or null)
+    int* Cs = nullptr;  // row-shifted copies of C for the tiled 2-opt (or null)
     uint16_t *X = nullptr, *V = nullptr, *P = nullptr, *G = nullptr;
     long long *F = nullptr, *PF = nullptr;
     unsigned long long* hash = nullptr;
@@ -315,8 +315,8 @@ int ensure_history(dpso_swarm* s, int need) {
     return DPSO_OK;
 }
 
-// The row-shifted copies of C that the tiled exchange kernels read: the node
-// swap's from the start, the 2-opt's when a batch pins a tiled shape.
+// The row-shifted copies of C that the tiled 2-opt kernel reads, made when a
+// batch pins a tiled shape.
 int ensure_shifted(dpso_swarm* s) {
     if (s->Cs) return DPSO_OK;
     const int n = s->k.n;
@@ -413,7 +413,7 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
                    int64_t* moves_host, void* stream) {
     if (!C_dev || !tours_dev || !cost_dev || n < 3 || count < 0 || max_moves < 0)
         return DPSO_ERR_ARG;
-    if (n > DPSO_MAX_N || (kind == 1 && node_swap_tiled_rows(n) == 0)) return DPSO_ERR_RANGE;
+    if (n > DPSO_MAX_N || (kind == 1 && !node_swap_fits(n))) return DPSO_ERR_RANGE;
     if (pairs_host) *pairs_host = 0;
     if (moves_host) *moves_host = 0;
     if (count == 0) return DPSO_OK;
@@ -447,23 +447,11 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    int* Cs = nullptr;
-    if (e == cudaSuccess && herr == 0 && kind == 1) {  // the node swap's row-shifted copies
-        if (cudaMallocAsync(&Cs, sizeof(int) * 4 * static_cast<size_t>(n) * shifted_ld(n), st) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            Cs = nullptr;
-            e = cudaErrorMemoryAllocation;
-        } else {
-            e = build_shifted_copies(C_dev, n, n, Cs, st);
-        }
-    }
     if (e == cudaSuccess && herr == 0) {
         e = launch_fitness(C_dev, n, n, tours_dev, n, count, reinterpret_cast<long long*>(cost_dev),
                            st);
         TwoOptTask& a = host.task;
         a.C = C_dev;
-        a.Cs = Cs;
         a.ldc = n;
         a.n = n;
         a.tours = tours_dev;
@@ -478,8 +466,7 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&scratch->task, &host.task, sizeof(TwoOptTask),
                                 cudaMemcpyHostToDevice, st);
-        TwoOptBatch tb{&scratch->task, scratch->toff, 1, count, n, Cs != nullptr, 0,
-                       &scratch->queue};
+        TwoOptBatch tb{&scratch->task, scratch->toff, 1, count, n, false, 0, &scratch->queue};
         tb.kind = kind;
         if (e == cudaSuccess) e = launch_two_opt(tb, sms, st);
         if (e == cudaSuccess)
@@ -489,7 +476,6 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host.task is read by the copy
     }
     cudaFreeAsync(scratch, st);
-    if (Cs) cudaFreeAsync(Cs, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaErrorMemoryAllocation) return DPSO_ERR_NO_MEMORY;
     if (e != cudaSuccess) return DPSO_ERR_CUDA;
@@ -562,7 +548,7 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
         cudaSuccess)
         return fail(DPSO_ERR_CUDA);
     const bool node_swap = (p->flags & DPSO_FLAG_TWO_OPT) && (p->flags & DPSO_FLAG_NODE_SWAP);
-    if (node_swap && node_swap_tiled_rows(n) == 0) return fail(DPSO_ERR_RANGE);
+    if (node_swap && !node_swap_fits(n)) return fail(DPSO_ERR_RANGE);
 
     Consts& k = s->k;
     k.n = n;
@@ -636,7 +622,6 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
         return fail2(DPSO_ERR_CUDA);
     if (herr & 1) return fail2(DPSO_ERR_ARG);
     if (herr & 2) return fail2(DPSO_ERR_RANGE);
-    if (node_swap && (st = ensure_shifted(s))) return fail2(st);
     {
         SwarmMeta m{};
         m.desc.k = k;
@@ -928,7 +913,7 @@ struct ShapeKey {
 ShapeKey default_shape(int n, int kind) {
     ShapeKey k;
     k.kind = kind;
-    if (kind == 1) k.cfg = node_swap_tiled_rows(n);  // one kernel shape per tile height
+    if (kind == 1) k.cfg = node_swap_class(n);
     else k.cfg = two_opt_class(n, &k.ctas);
     return k;
 }
@@ -994,7 +979,7 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
         tb = TwoOptBatch{cl.tasks, cl.toff, cnt, toff.back(), max_n, shifted, 0, cl.queue};
         tb.kind = keys[c].kind;
         if (keys[c].kind == 1) {
-            // node swap: the tile height follows max_n
+            // node swap: the launch follows max_n
         } else if (pinned) {
             tb.rows = pinned->rows;
             tb.tpc = pinned->tours_per_cta;

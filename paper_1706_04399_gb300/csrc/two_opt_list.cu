@@ -717,7 +717,7 @@ int two_opt_class(int n, int* ctas) {
 
 cudaError_t launch_two_opt(const TwoOptBatch& b, int num_sms, cudaStream_t st) {
     if (b.total <= 0) return cudaSuccess;
-    if (b.kind == 1) return launch_node_swap_tiled(b, num_sms, st);
+    if (b.kind == 1) return launch_node_swap(b, num_sms, st);
     if (b.rows > 0 && b.shifted) {  // a pinned shape of the tiled kernel
         const int tpc = b.tpc > 0 ? b.tpc : two_opt_tiled_tpc(b.max_n, b.rows);
         const int tg = b.tg > 0 ? b.tg : two_opt_tiled_tg(b.max_n, b.rows, tpc);
