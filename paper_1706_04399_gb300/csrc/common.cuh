@@ -110,8 +110,6 @@ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 // ---- launchers (cost.cu) ----
 cudaError_t launch_cost_matrix(const double* xyz, int n, const double* boxes, int m, double radius,
                                int penalty, int* C, int ldc, int* err, cudaStream_t st);
-cudaError_t launch_check_inputs(const double* xyz, int n, const double* boxes, int m, int* err,
-                                cudaStream_t st);
 cudaError_t launch_check_cost(const int* C, int n, int ldc, int* err, cudaStream_t st);
 cudaError_t launch_check_cost_limit(const int* C, int n, int ldc, int limit, int* err,
                                     cudaStream_t st);

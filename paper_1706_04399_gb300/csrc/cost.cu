@@ -5,6 +5,13 @@
 // Every FP64 step is an explicit round-to-nearest intrinsic, so nothing is
 // contracted into an FMA and sqrt / divide are the correctly rounded IEEE
 // operations; the file is also built with -fmad=false.
+//
+// FP64 is scarce here (about one multiply-add per SM and clock for each 32 in
+// FP32), and the slab test divides six times per pair and box.  A filter in
+// FP32 with an error bound decides nearly every (pair, box); the FP64 test runs
+// on what it leaves open, so the matrix is that of the FP64 test alone.  At
+// n = 1992 with 20 boxes the kernel takes 0.18 ms, 3.32 without the filter;
+// what is left is the FP64 distance and its square root, and the filter.
 #include <math.h>
 
 #include "common.cuh"
@@ -40,95 +47,201 @@ __device__ bool segment_blocked(const double p[3], const double q[3], const doub
 }
 
 constexpr int kTile = 32;
+constexpr int kBoxes = 256;  // boxes staged at once
 
-// One thread per (i, j) with i < j inside 32 x 32 tiles of the upper triangle;
-// boxes are staged in shared memory in chunks.
-__global__ void __launch_bounds__(kTile * 8) cost_matrix_kernel(
+// FP32 view of a pair on one axis: p, 1 / (q - p), and the smaller and larger
+// of p and q.
+struct Axis {
+    float p, inv, a, b;
+};
+
+// The FP32 filter for one box: 0 free, 1 blocked, 2 open.
+//
+// With M the largest magnitude of the pair's and the box's coordinates, every
+// difference of two of them is off by at most 2^-22 M (both rounded to FP32,
+// and the difference rounded); E is twice that and more.
+//  * An axis on which both ends lie E beyond the box: free.  (The FP64 test
+//    finds t > 1 or t < 0 there, by at least E / |d| >= 2^-22.)
+//  * An axis with |d| < 64 E, d = 0 among them: no constraint when both ends
+//    lie E inside, else open.
+//  * The other axes: t = (side - p) / d is off by at most E / |d| where it is
+//    near [0, 1], plus its own rounding; when the ends of the common interval
+//    are further apart than twice the largest such error, their order is that
+//    of the FP64 values, whose error is some 2^-52.
+// Infinities and NaN (coordinates past FP32) leave every comparison false: open.
+__device__ __forceinline__ int filter_box(const Axis (&ax)[3], const float (&lo)[3],
+                                          const float (&hi)[3], float E) {
+    bool out = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) out = out || ax[k].b < lo[k] - E || ax[k].a > hi[k] + E;
+    if (out) return 0;
+    float tmin = 0.f, tmax = 1.f, worst_inv = 0.f;
+    bool open = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (ax[k].b - ax[k].a >= 64.f * E) {
+            const float t1 = (lo[k] - ax[k].p) * ax[k].inv, t2 = (hi[k] - ax[k].p) * ax[k].inv;
+            tmin = fmaxf(tmin, fminf(t1, t2));
+            tmax = fminf(tmax, fmaxf(t1, t2));
+            worst_inv = fmaxf(worst_inv, fabsf(ax[k].inv));
+        } else {
+            open = open || !(ax[k].a > lo[k] + E && ax[k].b < hi[k] - E);
+        }
+    }
+    const float gap = tmax - tmin, w = 2.f * (E * worst_inv + 0x1p-19f);
+    if (gap < -w) return 0;
+    return !open && gap > w ? 1 : 2;
+}
+
+// One thread per (i, j) with i < j inside 32 x 32 tiles of the upper triangle,
+// four pairs per thread; boxes are staged in shared memory in chunks.  The
+// tile is mirrored through shared memory, so both halves are written in rows.
+// Flags non-finite coordinates and inverted boxes (bit 0 of *err) and entries
+// above DPSO_COST_MAX (bit 1).
+__global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
     const double* __restrict__ xyz, int n, const double* __restrict__ boxes, int m, double r,
     int penalty, int* __restrict__ C, int ldc, int* err) {
     const int bi = blockIdx.y * kTile, bj = blockIdx.x * kTile;
     if (bj + kTile <= bi) return;  // strictly below the diagonal
-    __shared__ double sbox[256 * 6];
+    __shared__ double sbox[kBoxes * 6];
+    __shared__ float slo[kBoxes][3], shi[kBoxes][3], smag[kBoxes];
+    __shared__ int tile[kTile][kTile + 1];
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-    long long base[4];
-    bool blocked[4];
-    int ii[4], jj[4];
-    double p[4][3], q[4][3];
+    const int tid = ty * kTile + tx;
+    const int j = bj + tx;
+    double q[3] = {0, 0, 0};
+    float qf[3];
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        ii[s] = bi + ty + 8 * s;
-        jj[s] = bj + tx;
-        blocked[s] = false;
-        base[s] = 0;
-        if (ii[s] < n && jj[s] < n && ii[s] < jj[s]) {
+    for (int k = 0; k < 3; ++k) {
+        if (j < n) q[k] = xyz[3 * (size_t)j + k];
+        qf[k] = static_cast<float>(q[k]);
+    }
+    bool bad = false;
+    unsigned blocked = 0;  // bit s: pair s
+    for (int b0 = 0; b0 < m; b0 += kBoxes) {
+        const int cnt = min(kBoxes, m - b0);
+        __syncthreads();
+        for (int e = tid; e < cnt * 6; e += kTile * 8) {
+            const double v = boxes[6 * (size_t)b0 + e];
+            sbox[e] = v;
+            bad = bad || !isfinite(v);
+        }
+        __syncthreads();
+        if (tid < cnt) {
+            float mg = 0.f;
+            for (int k = 0; k < 3; ++k) {
+                bad = bad || sbox[6 * tid + k] > sbox[6 * tid + 3 + k];
+                slo[tid][k] = static_cast<float>(__dsub_rn(sbox[6 * tid + k], r));
+                shi[tid][k] = static_cast<float>(__dadd_rn(sbox[6 * tid + 3 + k], r));
+                mg = fmaxf(mg, fmaxf(fabsf(slo[tid][k]), fabsf(shi[tid][k])));
+            }
+            smag[tid] = mg;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int s = 0; s < 4; ++s) {
+            const int i = bi + ty + 8 * s;
+            if (i >= n || j >= n || i >= j || (blocked >> s & 1)) continue;
+            double p[3];
+            Axis ax[3];
+            float mag = 0.f;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                p[s][k] = xyz[3 * (size_t)ii[s] + k];
-                q[s][k] = xyz[3 * (size_t)jj[s] + k];
+                p[k] = xyz[3 * (size_t)i + k];
+                const float pf = static_cast<float>(p[k]);
+                ax[k] = Axis{pf, 1.f / static_cast<float>(__dsub_rn(q[k], p[k])), fminf(pf, qf[k]),
+                             fmaxf(pf, qf[k])};
+                mag = fmaxf(mag, fmaxf(fabsf(pf), fabsf(qf[k])));
             }
-            const double dx = __dsub_rn(q[s][0], p[s][0]);
-            const double dy = __dsub_rn(q[s][1], p[s][1]);
-            const double dz = __dsub_rn(q[s][2], p[s][2]);
-            double acc = __dmul_rn(dx, dx);
-            acc = __dadd_rn(acc, __dmul_rn(dy, dy));
-            acc = __dadd_rn(acc, __dmul_rn(dz, dz));
-            base[s] = __double2ll_rn(__dmul_rn(1000.0, __dsqrt_rn(acc)));
+            bool hit = false;
+            for (int g0 = 0; g0 < cnt && !hit; g0 += 32) {
+                unsigned open = 0;
+                const int g1 = min(cnt, g0 + 32);
+#pragma unroll 2
+                for (int b = g0; b < g1; ++b) {
+                    const float lo[3] = {slo[b][0], slo[b][1], slo[b][2]};
+                    const float hi[3] = {shi[b][0], shi[b][1], shi[b][2]};
+                    const int v = filter_box(ax, lo, hi, (mag + smag[b]) * 0x1p-20f + 1e-30f);
+                    hit = hit || v == 1;
+                    open |= static_cast<unsigned>(v == 2) << (b - g0);
+                }
+                for (; open && !hit; open &= open - 1)
+                    hit = segment_blocked(p, q, sbox + 6 * (g0 + __ffs(open) - 1), r);
+            }
+            blocked |= static_cast<unsigned>(hit) << s;
         }
     }
-    for (int b0 = 0; b0 < m; b0 += 256) {
-        const int cnt = min(256, m - b0);
-        __syncthreads();
-        for (int e = ty * kTile + tx; e < cnt * 6; e += kTile * 8) sbox[e] = boxes[6 * (size_t)b0 + e];
-        __syncthreads();
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            if (ii[s] < n && jj[s] < n && ii[s] < jj[s]) {
-                for (int b = 0; b < cnt && !blocked[s]; ++b)
-                    blocked[s] = segment_blocked(p[s], q[s], sbox + 6 * b, r);
-            }
-        }
-    }
+    int vals[4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-        const int i = ii[s], j = jj[s];
-        if (i >= n || j >= n) continue;
-        if (i == j) {
-            C[(size_t)i * ldc + i] = 0;
-            continue;
+        const int i = bi + ty + 8 * s;
+        vals[s] = 0;
+        if (i >= n) continue;
+        double p[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            p[k] = xyz[3 * (size_t)i + k];
+            bad = bad || !isfinite(p[k]);  // (every point is a row of its diagonal tile)
         }
-        if (i > j) continue;
-        long long v = base[s] + (blocked[s] ? (long long)penalty : 0LL);
-        if (v > DPSO_COST_MAX) {
+        if (j >= n || i >= j) continue;
+        const double dx = __dsub_rn(q[0], p[0]);
+        const double dy = __dsub_rn(q[1], p[1]);
+        const double dz = __dsub_rn(q[2], p[2]);
+        double acc = __dmul_rn(dx, dx);
+        acc = __dadd_rn(acc, __dmul_rn(dy, dy));
+        acc = __dadd_rn(acc, __dmul_rn(dz, dz));
+        long long c = __double2ll_rn(__dmul_rn(1000.0, __dsqrt_rn(acc))) +
+                      ((blocked >> s & 1) ? (long long)penalty : 0LL);
+        if (c > DPSO_COST_MAX) {
             atomicOr(err, 2);
-            v = DPSO_COST_MAX;
+            c = DPSO_COST_MAX;
         }
-        C[(size_t)i * ldc + j] = static_cast<int>(v);
-        C[(size_t)j * ldc + i] = static_cast<int>(v);
+        vals[s] = static_cast<int>(c);
     }
-}
-
-// Flags non-finite coordinates and inverted boxes (bit 0 of *err).
-__global__ void check_inputs_kernel(const double* __restrict__ xyz, int n,
-                                    const double* __restrict__ boxes, int m, int* err) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < 3 * n && !isfinite(xyz[k])) atomicOr(err, 1);
-    if (k < m) {
-        for (int a = 0; a < 6; ++a)
-            if (!isfinite(boxes[6 * (size_t)k + a])) atomicOr(err, 1);
-        for (int a = 0; a < 3; ++a)
-            if (boxes[6 * (size_t)k + a] > boxes[6 * (size_t)k + 3 + a]) atomicOr(err, 1);
+    if (bad) atomicOr(err, 1);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int i = bi + ty + 8 * s;
+        if (i < n && j < n && i <= j) C[(size_t)i * ldc + j] = vals[s];  // (0 on the diagonal)
+        tile[ty + 8 * s][tx] = vals[s];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {  // row bj + r of the lower half, columns bi ..
+        const int rr = ty + 8 * s, row = bj + rr, col = bi + tx;
+        if (row < n && col < n && col < row) C[(size_t)row * ldc + col] = tile[tx][rr];
     }
 }
 
 // Flags an asymmetric matrix or a non-zero diagonal (bit 0) and entries outside
-// [0, limit] (bit 1).
-__global__ void check_cost_kernel(const int* __restrict__ C, int n, int ldc, int limit, int* err) {
-    const int i = blockIdx.y;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const int v = C[(size_t)i * ldc + j];
-        if (v < 0 || v > limit) atomicOr(err, 2);
-        if (i == j ? v != 0 : v != C[(size_t)j * ldc + i]) atomicOr(err, 1);
+// [0, limit] (bit 1).  A block compares a 32 x 32 tile on or above the diagonal
+// with its mirror image, read in rows and turned in shared memory: bound by the
+// one read of the matrix (read down columns instead, it took 20 us at
+// n = 1992).
+__global__ void __launch_bounds__(kTile * 8) check_cost_kernel(const int* __restrict__ C, int n,
+                                                               int ldc, int limit, int* err) {
+    const int bi = blockIdx.y * kTile, bj = blockIdx.x * kTile;
+    if (bj < bi) return;
+    __shared__ int tile[kTile][kTile + 1];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    int bits = 0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {  // the mirror tile
+        const int i = bj + ty + 8 * s, j = bi + tx;
+        const int v = i < n && j < n ? C[(size_t)i * ldc + j] : 0;
+        if (v < 0 || v > limit) bits |= 2;
+        tile[ty + 8 * s][tx] = v;
     }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int i = bi + ty + 8 * s, j = bj + tx;
+        if (i >= n || j >= n) continue;
+        const int v = C[(size_t)i * ldc + j];
+        if (v < 0 || v > limit) bits |= 2;
+        if (i == j ? v != 0 : v != tile[tx][ty + 8 * s]) bits |= 1;
+    }
+    if (bits) atomicOr(err, bits);
 }
 
 }  // namespace
@@ -141,21 +254,14 @@ cudaError_t launch_cost_matrix(const double* xyz, int n, const double* boxes, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_check_inputs(const double* xyz, int n, const double* boxes, int m, int* err,
-                                cudaStream_t st) {
-    const int work = max(3 * n, m);
-    check_inputs_kernel<<<(work + 255) / 256, 256, 0, st>>>(xyz, n, boxes, m, err);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_check_cost(const int* C, int n, int ldc, int* err, cudaStream_t st) {
     return launch_check_cost_limit(C, n, ldc, DPSO_COST_MAX, err, st);
 }
 
 cudaError_t launch_check_cost_limit(const int* C, int n, int ldc, int limit, int* err,
                                     cudaStream_t st) {
-    dim3 grid((n + 255) / 256, n);
-    check_cost_kernel<<<grid, 256, 0, st>>>(C, n, ldc, limit, err);
+    const int tiles = (n + kTile - 1) / kTile;
+    check_cost_kernel<<<dim3(tiles, tiles), dim3(kTile, 8), 0, st>>>(C, n, ldc, limit, err);
     return cudaGetLastError();
 }
 
@@ -176,7 +282,6 @@ extern "C" int dpso_cost_matrix(const double* xyz_dev, int32_t n, const double* 
     if (cudaMallocAsync(&err, sizeof(int), st) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
     int herr = 0;
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = launch_check_inputs(xyz_dev, n, boxes_dev, m, err, st);
     if (e == cudaSuccess)
         e = launch_cost_matrix(xyz_dev, n, boxes_dev, m, cp->uav_radius_m, cp->blocked_penalty_mm,
                                C_dev, n, err, st);
