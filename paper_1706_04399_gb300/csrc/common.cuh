@@ -130,7 +130,7 @@ struct BatchView {
     int ninst;
     int total;    // off[ninst]: particles in the batch
     int max_ldn;  // largest ldn: sizes the move kernel's shared memory
-    int arrays;   // shared arrays per particle in the move kernel: 7 if any w < 1, else 5
+    int arrays;   // shared arrays per particle in the move kernel: 8 if any w < 1, else 7
     int max_S;    // largest swarm of the batch
 };
 

@@ -171,7 +171,7 @@ TwoOptTask swarm_task(const dpso_swarm* s) {
     return a;
 }
 
-int swarm_arrays(const Consts& k) { return k.w_q >= (1ull << 32) ? 5 : 7; }
+int swarm_arrays(const Consts& k) { return k.w_q >= (1ull << 32) ? 7 : 8; }
 
 BatchView swarm_view(const dpso_swarm* s) {
     return BatchView{&s->meta->desc, s->meta->off, 1, s->k.S, s->k.ldn, swarm_arrays(s->k), s->k.S};
@@ -204,7 +204,8 @@ cudaError_t enqueue_generation(dpso_swarm* s, bool mut_iter, cudaStream_t st,
     if (e == cudaSuccess) e = mark(2);
     if (e == cudaSuccess) e = launch_gbest(bv, 0, st);
     if (e == cudaSuccess) e = mark(3);
-    if (e == cudaSuccess && two) e = launch_rank_cost(bv, st);
+    // (with a tour per SM at most all start at once, in whatever order)
+    if (e == cudaSuccess && two && s->k.S > s->num_sms) e = launch_rank_cost(bv, st);
     if (e == cudaSuccess && two) e = cudaMemsetAsync(tb.queue, 0, sizeof(unsigned int), st);
     if (e == cudaSuccess && two) e = launch_two_opt(tb, s->num_sms, st);
     if (e == cudaSuccess) e = mark(4);
@@ -246,7 +247,7 @@ int collect_timing(dpso_swarm* s) {
         s->acc.ms[DPSO_PHASE_GBEST] += t[2] + t[4];
         s->acc.ms[DPSO_PHASE_TWO_OPT] += t[3];
         s->acc.launches[DPSO_PHASE_MOVE] += 1;
-        s->acc.launches[DPSO_PHASE_MUTATION] += pr[1] ? 4 : 0;
+        s->acc.launches[DPSO_PHASE_MUTATION] += pr[1] ? 3 : 0;
         s->acc.launches[DPSO_PHASE_GBEST] += two ? 2 : 1;
         s->acc.launches[DPSO_PHASE_TWO_OPT] += two ? 1 : 0;
         s->acc.generations += 1;
@@ -1008,7 +1009,7 @@ cudaError_t enqueue_batch_classes(dpso_batch* b, cudaStream_t st) {
     if (e == cudaSuccess) e = launch_mutation(b->bv, st);
     if (e == cudaSuccess) e = launch_gbest(b->bv, 0, st);
     if (e != cudaSuccess || !b->any_two_opt) return e;
-    e = launch_rank_cost(b->bv, st);
+    if (b->bv.total > b->num_sms) e = launch_rank_cost(b->bv, st);
     if (e == cudaSuccess && b->cls.size() > 1) e = cudaEventRecord(b->ev[0], st);
     for (size_t c = 1; c < b->cls.size() && e == cudaSuccess; ++c) {
         cudaStream_t s = b->side[c - 1];
@@ -1175,7 +1176,7 @@ int dpso_batch_create(dpso_batch** out, dpso_swarm* const* swarms, int32_t count
         return fail(DPSO_ERR_CUDA);
     std::vector<SwarmDesc> desc(count);
     std::vector<int> off(count + 1, 0);
-    int max_ldn = 0, max_S = 0, arrays = 5;
+    int max_ldn = 0, max_S = 0, arrays = 7;
     for (int i = 0; i < count; ++i) {
         const dpso_swarm* s = swarms[i];
         desc[i].k = s->k;

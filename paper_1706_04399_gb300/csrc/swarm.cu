@@ -99,10 +99,12 @@ __device__ __forceinline__ bool key_less(const Key& a, const Key& b) {
     return a.pos < b.pos;
 }
 
-__global__ void det_orders_kernel(const int* __restrict__ tags, int n, uint16_t* orders, int ldn,
-                                  int* err) {
-    const int v = blockIdx.y;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Eight lanes count one viewpoint's rank, each over every eighth viewpoint: 38
+// us at n = 1992 (243 with one thread per viewpoint).
+__global__ void __launch_bounds__(256) det_orders_kernel(const int* __restrict__ tags, int n,
+                                                         uint16_t* orders, int ldn, int* err) {
+    const int v = blockIdx.y, part = threadIdx.x & 7;
+    const int i = blockIdx.x * 32 + (threadIdx.x >> 3);
     __shared__ int st[3 * 512];
     Key mine{0, 0, 0};
     if (i < n) mine = det_key(tags, i, v);
@@ -112,15 +114,19 @@ __global__ void det_orders_kernel(const int* __restrict__ tags, int n, uint16_t*
         __syncthreads();
         for (int e = threadIdx.x; e < 3 * cnt; e += blockDim.x) st[e] = tags[3 * j0 + e];
         __syncthreads();
-        if (i < n) {
-            for (int j = 0; j < cnt; ++j) {
-                const Key o = det_key(st, j, v);
-                rank += key_less(o, mine);
-                same += !key_less(o, mine) && !key_less(mine, o);
-            }
+#pragma unroll 4
+        for (int j = part; j < cnt; j += 8) {
+            const Key o = det_key(st, j, v);
+            rank += key_less(o, mine);
+            same += o.face == mine.face && o.line == mine.line && o.pos == mine.pos;
         }
     }
-    if (i < n) {
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        rank += __shfl_xor_sync(kFull, rank, o);
+        same += __shfl_xor_sync(kFull, same, o);
+    }
+    if (i < n && part == 0) {
         if (same != 1) atomicOr(err, 1);
         else orders[(size_t)v * ldn + rank] = static_cast<uint16_t>(i);
     }
@@ -132,36 +138,54 @@ __global__ void det_orders_kernel(const int* __restrict__ tags, int n, uint16_t*
 // (n-1-i) of phase 1 bounded to [0, i], swap x[i], x[j].  v = identity,
 // pbest = x.
 
-__global__ void init_particles_kernel(Consts k, SwarmDev d, const uint16_t* __restrict__ orders,
-                                      int n_det) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= k.S) return;
-    const int n = k.n;
+// One warp per particle.  The draws are taken by all lanes; the swaps are one
+// chain, run by lane 0 in shared memory: 43 us for 512 particles at n = 1992
+// (1085 with one thread per particle on global memory).
+__global__ void __launch_bounds__(32) init_particles_kernel(Consts k, SwarmDev d,
+                                                            const uint16_t* __restrict__ orders,
+                                                            int n_det) {
+    extern __shared__ __align__(16) uint16_t sm[];
+    const int p = blockIdx.x, lane = threadIdx.x, n = k.n;
     uint16_t* x = d.X + (size_t)p * k.ldn;
+    uint16_t* pb = d.P + (size_t)p * k.ldn;
+    uint16_t* v = d.V + (size_t)p * k.ldn;
+    uint16_t* y = sm;            // the permutation
+    uint16_t* with = sm + k.ldn;  // swap partner of position i
     if (p < n_det) {
         const uint16_t* ord = orders + (size_t)(p % 8) * k.ldn;
         const int rot = (p / 8) % n;
-        for (int i = 0; i < n; ++i) x[i] = ord[(i + rot) % n];
+        for (int i = lane; i < n; i += 32) {
+            const int at = i + rot;
+            y[i] = ord[at < n ? at : at - n];
+        }
     } else {
-        for (int i = 0; i < n; ++i) x[i] = static_cast<uint16_t>(i);
-        for (int d0 = 0; d0 < n - 1; d0 += 4) {
-            const Block4 b = philox(static_cast<uint32_t>(d0 >> 2), p, 0, kPhaseInit, k.seed);
+        for (int i = lane; i < n; i += 32) y[i] = static_cast<uint16_t>(i);
+        for (int b0 = lane; 4 * b0 < n - 1; b0 += 32) {
+            const Block4 b = philox(static_cast<uint32_t>(b0), p, 0, kPhaseInit, k.seed);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int dd = d0 + q;
-                if (dd >= n - 1) break;
-                const int i = n - 1 - dd;
-                const int j = static_cast<int>(bounded(b.v[q], static_cast<uint32_t>(i + 1)));
-                const uint16_t tmp = x[i];
-                x[i] = x[j];
-                x[j] = tmp;
+                const int i = n - 1 - (4 * b0 + q);
+                if (i > 0)
+                    with[i] = static_cast<uint16_t>(bounded(b.v[q], static_cast<uint32_t>(i + 1)));
+            }
+        }
+        __syncwarp();
+        if (lane == 0) {
+            int j = with[n - 1];
+            for (int i = n - 1; i > 0; --i) {
+                const int nxt = with[i - 1];
+                const uint16_t a = y[i], b = y[j];
+                y[i] = b;
+                y[j] = a;
+                j = nxt;
             }
         }
     }
-    uint16_t* pb = d.P + (size_t)p * k.ldn;
-    uint16_t* v = d.V + (size_t)p * k.ldn;
-    for (int i = 0; i < n; ++i) {
-        pb[i] = x[i];
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
+        const uint16_t yi = y[i];
+        x[i] = yi;
+        pb[i] = yi;
         v[i] = static_cast<uint16_t>(i);
     }
 }
@@ -212,37 +236,90 @@ __global__ void gbest_init_kernel(Consts k, SwarmDev d) {
 }
 
 // ---------------------------------------------------------------- the move
-// Sec. 3.1 subtraction x2 - x1 read as the greedy left-to-right list: scan
-// positions, and where the running copy y differs from the target, swap the
-// labels y[k] and tgt[k] (found through the inverse map pos).  The swap is
-// written branch-free; when y[k] == tgt[k] it stores the same values back.
-// Stops after `limit` transpositions; returns how many were applied.  tgt is
-// read in 16-byte chunks (rows are padded to multiples of 8 labels).
-__device__ int greedy_subtract(uint16_t* y, uint16_t* pos, const uint16_t* __restrict__ tgt,
-                               int n, int limit) {
-    int cnt = 0;
-    if (limit <= 0) return 0;
-    uint4 cur = *reinterpret_cast<const uint4*>(tgt);
-    for (int k0 = 0; k0 < n; k0 += 8) {
-        const uint4 nxt = (k0 + 8 < n) ? *reinterpret_cast<const uint4*>(tgt + k0 + 8) : cur;
-        const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w};
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int kk = k0 + q;
-            if (kk >= n) break;
-            const uint16_t b = static_cast<uint16_t>(w[q >> 1] >> ((q & 1) * 16));
-            const uint16_t a = y[kk];
-            const uint16_t pb = pos[b];
-            y[kk] = b;
-            y[pb] = a;
-            pos[b] = static_cast<uint16_t>(kk);
-            pos[a] = pb;
-            cnt += (a != b);
-            if (cnt >= limit) return cnt;
+// Sec. 3.1 subtraction tgt - base read as the greedy left-to-right list: scan
+// positions; where the running copy y differs from the target, swap the labels
+// y[k] and tgt[k].  Written out, the list is a chain of n dependent steps; its
+// effect is not.  With next(c) the place in the target of the label at
+// position c of the base, the cycles of `next` are what the list sorts:
+//  * Step k swaps unless k is the last place of its cycle that the scan
+//    reaches, its largest; so the list has n - cycles transpositions, and the
+//    first `cnt` of them end at the place K - 1 of the cnt-th k that is not
+//    the largest of its cycle.
+//  * After them y[k] = tgt[k] below K; at and past K, y[k] is the label at the
+//    end of the chain k, next(k), next(next(k)), .. that runs through places
+//    below K, i.e. the first c whose next(c) is not below K.
+// Both are found by doubling: each round every place joins the stretch of its
+// path it knows with the stretch that starts where its own ends (a place's
+// end and largest member share a word, so a round may run in place).
+
+// |tgt - base| and, with `next` left in `nxt`, what truncation needs: low half
+// of big[c] unused afterwards, high half the largest place of c's cycle.
+__device__ int subtract_cycles(const uint16_t* ix, const uint16_t* tgt, uint16_t* nxt,
+                               uint32_t* big, int n, int lane) {
+    for (int k = lane; k < n; k += 32) nxt[ix ? ix[tgt[k]] : tgt[k]] = static_cast<uint16_t>(k);
+    __syncwarp();
+    for (int c = lane; c < n; c += 32) big[c] = (static_cast<uint32_t>(c) << 16) | nxt[c];
+    __syncwarp();
+    for (int known = 1; known < n; known *= 2) {
+        for (int c = lane; c < n; c += 32) {
+            const uint32_t a = big[c], b = big[a & 0xffffu];
+            big[c] = (max(a >> 16, b >> 16) << 16) | (b & 0xffffu);
         }
-        cur = nxt;
+        __syncwarp();
     }
-    return cnt;
+    int cnt = 0;
+    for (int c = lane; c < n; c += 32) cnt += (big[c] >> 16) != static_cast<uint32_t>(c);
+    return __reduce_add_sync(kFull, cnt);
+}
+
+// y = base after the first `cnt` of the `len` transpositions of tgt - base
+// (base: x, or the identity when x is null); uses and overwrites nxt.
+__device__ void subtract_apply(const uint16_t* x, const uint16_t* tgt, uint16_t* nxt,
+                               const uint32_t* big, int cnt, int len, uint16_t* y, int n,
+                               int lane) {
+    int K = cnt >= len ? n : 0;
+    if (cnt < len && cnt > 0) {
+        int seen = 0;
+        for (int c0 = 0; c0 < n; c0 += 32) {
+            const int c = c0 + lane;
+            const unsigned mask =
+                __ballot_sync(kFull, c < n && (big[c] >> 16) != static_cast<uint32_t>(c));
+            const int here = __popc(mask);
+            if (seen + here >= cnt) {
+                K = c0 + __fns(mask, 0, cnt - seen) + 1;
+                break;
+            }
+            seen += here;
+        }
+    }
+    if (K > 0 && K < n) {
+        // (a cycle that lies wholly below K has no end and is not asked for)
+        for (int c = lane; c < n; c += 32) {
+            const int t = nxt[c], top = static_cast<int>(big[c] >> 16);
+            nxt[c] = static_cast<uint16_t>(t >= K || top < K ? c : t);
+        }
+        __syncwarp();
+        bool moved = true;  // a chain has fewer than n places: log2 n rounds at most
+        for (int known = 1; known < n && moved; known *= 2) {
+            bool mine = false;
+            for (int c = lane; c < n; c += 32) {
+                const uint16_t t = nxt[c], u = nxt[t];
+                mine = mine || t != u;
+                nxt[c] = u;
+            }
+            __syncwarp();
+            moved = __any_sync(kFull, mine);
+        }
+    }
+    for (int k = lane; k < n; k += 32) {
+        if (k < K) {
+            y[k] = tgt[k];
+        } else {
+            const uint16_t c = K > 0 ? nxt[k] : static_cast<uint16_t>(k);
+            y[k] = x ? x[c] : c;
+        }
+    }
+    __syncwarp();
 }
 
 // floor(c |v|) with c = phi * u / 2^32 in Q32 fixed point.
@@ -251,19 +328,22 @@ __device__ __forceinline__ int scaled_count(unsigned long long phi_q, uint32_t u
     return static_cast<int>((cq * static_cast<unsigned long long>(len)) >> 32);
 }
 
-// One warp per particle.  Shared memory per warp: ya/pa (copy of x moved
-// toward P and its inverse), yb/pb (toward G), ix (inverse of x) and, when
-// w < 1, yw/pw (identity moved toward the velocity permutation).
-//   1. full greedy passes give |P - x|, |G - x| (and |v|): lanes 0, 1 (2)
-//   2. truncated passes apply the first ka / kb (kw) transpositions
-//   3. v <- sigma_b o sigma_a o sigma_wv, x <- v o x, fitness, pbest
-// One warp per particle of any instance in the batch.  Shared memory per
-// warp: ya/pa (copy of x moved toward P and its inverse), yb/pb (toward G),
-// ix (inverse of x) and, when the instance has w < 1, yw/pw (identity moved
-// toward the velocity permutation).
-//   1. full greedy passes give |P - x|, |G - x| (and |v|): lanes 0, 1 (2)
-//   2. truncated passes apply the first ka / kb (kw) transpositions
-//   3. v <- sigma_b o sigma_a o sigma_wv, x <- v o x, fitness, pbest
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
+    z += 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
+// One warp per particle of any instance in the batch: the truncated
+// subtractions toward P and G (and of the velocity from the identity when the
+// instance has w < 1) in shared memory, then v <- sigma_b o sigma_a o
+// sigma_wv, x <- v o x, fitness, pbest, and in mutation generations the hash
+// of the new tour.  Shared memory per warp: xs (x), ix (its inverse), nxt, ya,
+// yb (x moved toward P and G) and big; with w < 1 also yw.  What bounds it:
+// the log2 n rounds of the cycle search, shared-memory loads in random order:
+// 167 us for 512 particles at n = 1992, 39 us for 1024 at n = 400 (the list
+// run step by step by one lane: 343 and 78).
 __global__ void move_kernel(BatchView b) {
     extern __shared__ __align__(16) uint16_t sm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -278,77 +358,72 @@ __global__ void move_kernel(BatchView b) {
     const int t = ctl->t + 1;
     const int n = k.n, ldn = k.ldn;
     const bool partial = k.w_q < (1ull << 32);
-    uint16_t* ya = sm + static_cast<size_t>(warp) * b.arrays * b.max_ldn;
-    uint16_t* pa = ya + ldn;
-    uint16_t* yb = pa + ldn;
-    uint16_t* pb = yb + ldn;
-    uint16_t* ix = pb + ldn;
-    uint16_t* yw = ix + ldn;
-    uint16_t* pw = yw + ldn;
+    uint16_t* xs = sm + static_cast<size_t>(warp) * b.arrays * b.max_ldn;
+    uint32_t* big = reinterpret_cast<uint32_t*>(xs);  // two arrays wide
+    xs += 2 * ldn;
+    uint16_t* ix = xs + ldn;
+    uint16_t* nxt = ix + ldn;
+    uint16_t* ya = nxt + ldn;
+    uint16_t* yb = ya + ldn;
+    uint16_t* yw = yb + ldn;
     uint16_t* x = d.X + static_cast<size_t>(p) * ldn;
     uint16_t* v = d.V + static_cast<size_t>(p) * ldn;
     uint16_t* P = d.P + static_cast<size_t>(p) * ldn;
-    const uint16_t* G = d.G;
-    const int lanes = partial ? (k.w_q == 0 ? 2 : 3) : 2;
 
-    auto reset = [&]() {
-        for (int i = lane; i < n; i += 32) {
-            const uint16_t xi = x[i];
-            ix[xi] = static_cast<uint16_t>(i);
-            ya[i] = xi;
-            pa[xi] = static_cast<uint16_t>(i);
-            yb[i] = xi;
-            pb[xi] = static_cast<uint16_t>(i);
-            if (partial) {
-                yw[i] = static_cast<uint16_t>(i);
-                pw[i] = static_cast<uint16_t>(i);
-            }
+    for (int i = lane; i < n; i += 32) {
+        const uint16_t xi = x[i];
+        xs[i] = xi;
+        ix[xi] = static_cast<uint16_t>(i);
+    }
+    __syncwarp();
+    const Block4 r = philox(0, p, t, kPhaseVelocity, k.seed);
+    {
+        const int len = subtract_cycles(ix, P, nxt, big, n, lane);
+        subtract_apply(xs, P, nxt, big, scaled_count(k.phi1_q, r.v[0], len), len, ya, n, lane);
+    }
+    {
+        const int len = subtract_cycles(ix, d.G, nxt, big, n, lane);
+        subtract_apply(xs, d.G, nxt, big, scaled_count(k.phi2_q, r.v[1], len), len, yb, n, lane);
+    }
+    if (partial) {
+        if (k.w_q == 0) {
+            for (int l = lane; l < n; l += 32) yw[l] = static_cast<uint16_t>(l);
+        } else {
+            const int len = subtract_cycles(nullptr, v, nxt, big, n, lane);
+            const int kw = static_cast<int>((k.w_q * static_cast<unsigned long long>(len)) >> 32);
+            subtract_apply(nullptr, v, nxt, big, kw, len, yw, n, lane);
         }
         __syncwarp();
-    };
-    auto run = [&](int lim_a, int lim_b, int lim_w) {
-        int c = 0;
-        if (lane == 0) c = greedy_subtract(ya, pa, P, n, lim_a);
-        else if (lane == 1) c = greedy_subtract(yb, pb, G, n, lim_b);
-        else if (lane == 2 && lanes == 3) c = greedy_subtract(yw, pw, v, n, lim_w);
-        __syncwarp();
-        return c;
-    };
+    }
 
-    reset();
-    const int c0 = run(n, n, n);
-    const int La = __shfl_sync(kFull, c0, 0), Lb = __shfl_sync(kFull, c0, 1);
-    const int Lw = __shfl_sync(kFull, c0, 2);
-    const Block4 r = philox(0, p, t, kPhaseVelocity, k.seed);
-    const int ka = scaled_count(k.phi1_q, r.v[0], La);
-    const int kb = scaled_count(k.phi2_q, r.v[1], Lb);
-    const int kw = partial ? static_cast<int>(
-                                 (k.w_q * static_cast<unsigned long long>(lanes == 3 ? Lw : 0)) >> 32)
-                           : 0;
-    reset();
-    run(ka, kb, kw);
-
-    // sigma_a(m) = ya[ix[m]], sigma_b(m) = yb[ix[m]]; new velocity into pa.
+    // sigma_a(m) = ya[ix[m]], sigma_b(m) = yb[ix[m]]; new velocity into nxt.
     for (int l = lane; l < n; l += 32) {
         uint16_t m = partial ? yw[l] : v[l];
         m = ya[ix[m]];
         m = yb[ix[m]];
-        pa[l] = m;
+        nxt[l] = m;
+        v[l] = m;
     }
     __syncwarp();
-    for (int l = lane; l < n; l += 32) v[l] = pa[l];
+    const bool hashed = mutation_due(k, ctl);
+    unsigned long long h = 0;
     for (int i = lane; i < n; i += 32) {
-        const uint16_t xn = pa[x[i]];
-        pb[i] = xn;
+        const uint16_t xn = nxt[xs[i]];
+        ya[i] = xn;
         x[i] = xn;
+        if (hashed) h += mix64((static_cast<unsigned long long>(i) << 16) | xn);
     }
     __syncwarp();
-    const long long f = tour_cost_warp(d.C, k.ldc, n, pb, lane);
+    const long long f = tour_cost_warp(d.C, k.ldc, n, ya, lane);
+    if (hashed) {
+        h = warp_sum_u(h);
+        if (lane == 0) d.hash[p] = h;
+    }
     const long long pf = d.PF[p];  // read by every lane before lane 0 may write it
     __syncwarp();
     if (lane == 0) d.F[p] = f;
     if (f < pf) {
-        for (int i = lane; i < n; i += 32) P[i] = pb[i];
+        for (int i = lane; i < n; i += 32) P[i] = ya[i];
         if (lane == 0) d.PF[p] = f;
     }
 }
@@ -360,14 +435,7 @@ __global__ void move_kernel(BatchView b) {
 // swaps of two distinct positions (phase-3 draws 2q, 2q+1), an empty
 // velocity, a new fitness and a pbest update.  Equal tours have equal
 // fitness, so "earlier" means equal fitness and a smaller index; a 64-bit
-// hash screens the candidates and full compares decide.
-
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-    z += 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
+// hash (the move kernel's) screens the candidates and full compares decide.
 
 // Global particle g of the batch -> (instance, particle); false when g is past
 // the batch or the instance does not mutate in its running generation.
@@ -381,20 +449,6 @@ __device__ __forceinline__ bool mut_item(const BatchView& b, int g, Consts& k, S
     return mutation_due(k, d.ctl);
 }
 
-__global__ void mut_hash_kernel(BatchView b) {
-    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    Consts k;
-    SwarmDev d;
-    int p;
-    if (!mut_item(b, g, k, d, p)) return;
-    const uint16_t* x = d.X + static_cast<size_t>(p) * k.ldn;
-    unsigned long long h = 0;
-    for (int i = lane; i < k.n; i += 32)
-        h += mix64((static_cast<unsigned long long>(i) << 16) | x[i]);
-    h = warp_sum_u(h);
-    if (lane == 0) d.hash[p] = h;
-}
-
 __device__ bool tours_equal(const uint16_t* a, const uint16_t* b, int ldn) {
     const uint4* va = reinterpret_cast<const uint4*>(a);
     const uint4* vb = reinterpret_cast<const uint4*>(b);
@@ -405,35 +459,39 @@ __device__ bool tours_equal(const uint16_t* a, const uint16_t* b, int ldn) {
     return true;
 }
 
+// One warp per particle, the lanes over the others: 12 and 15 us for 1024
+// particles in this kernel and the next (83 and 91 with one thread each).
 __global__ void mut_dup_kernel(BatchView b) {
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     Consts k;
     SwarmDev d;
     int p;
-    if (!mut_item(b, blockIdx.x * blockDim.x + threadIdx.x, k, d, p)) return;
+    if (!mut_item(b, g, k, d, p)) return;
     const long long fp = d.F[p];
     const unsigned long long hp = d.hash[p];
-    unsigned char dup = 0;
-    for (int q = 0; q < p && !dup; ++q)
+    bool dup = false;
+#pragma unroll 4
+    for (int q = lane; q < p; q += 32)
         if (d.F[q] == fp && d.hash[q] == hp)
-            dup = tours_equal(d.X + static_cast<size_t>(q) * k.ldn,
-                              d.X + static_cast<size_t>(p) * k.ldn, k.ldn);
-    d.dup[p] = dup;
+            dup = dup || tours_equal(d.X + static_cast<size_t>(q) * k.ldn,
+                                     d.X + static_cast<size_t>(p) * k.ldn, k.ldn);
+    dup = __any_sync(kFull, dup);
+    if (lane == 0) d.dup[p] = dup;
 }
 
 __global__ void mut_kept_kernel(BatchView b) {
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     Consts k;
     SwarmDev d;
     int p;
-    if (!mut_item(b, blockIdx.x * blockDim.x + threadIdx.x, k, d, p)) return;
-    unsigned char kept = 0;
-    if (!d.dup[p]) {
-        const long long fp = d.F[p];
-        int rank = 0;
-        for (int q = 0; q < k.S; ++q)
-            rank += !d.dup[q] && (d.F[q] < fp || (d.F[q] == fp && q < p));
-        kept = rank < (k.S + 2) / 3;
-    }
-    d.kept[p] = kept;
+    if (!mut_item(b, g, k, d, p)) return;
+    const long long fp = d.F[p];
+    int rank = 0;
+#pragma unroll 4
+    for (int q = lane; q < k.S; q += 32)
+        rank += !d.dup[q] && (d.F[q] < fp || (d.F[q] == fp && q < p));
+    rank = __reduce_add_sync(kFull, rank);
+    if (lane == 0) d.kept[p] = !d.dup[p] && rank < (k.S + 2) / 3;
 }
 
 __global__ void mut_apply_kernel(BatchView b) {
@@ -520,31 +578,24 @@ __global__ void gbest_kernel(BatchView b, int second) {
 // order[r] = the particle of rank r by (fitness descending, index ascending)
 // within each instance, so the edge exchange starts the tours expected to
 // need the most passes first (longest-processing-time-first list
-// scheduling; the post-move fitness is the estimate).  Block (x, y) ranks
-// particles x*256 .. x*256+255 of instance y against all of its particles.
+// scheduling; the post-move fitness is the estimate).  One warp per particle:
+// 6 us for 1024 (17 with one thread each).
 __global__ void rank_cost_kernel(BatchView b) {
-    const int inst = blockIdx.y;
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (g >= b.total) return;
+    const int inst = find_inst(b.off, b.ninst, g);
     const SwarmDesc& ds = b.desc[inst];
-    const int S = ds.k.S;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x * blockDim.x >= S) return;  // whole block past this swarm
+    const int p = g - b.off[inst], S = ds.k.S;
     const long long* __restrict__ F = ds.d.F;
-    __shared__ long long sf[256];
-    const long long mine = p < S ? F[p] : 0;
+    const long long mine = F[p];
     int rank = 0;
-    for (int q0 = 0; q0 < S; q0 += 256) {
-        const int cnt = min(256, S - q0);
-        __syncthreads();
-        if (threadIdx.x < cnt) sf[threadIdx.x] = F[q0 + threadIdx.x];
-        __syncthreads();
-        if (p < S) {
-            for (int j = 0; j < cnt; ++j) {
-                const long long o = sf[j];
-                rank += (o > mine) | ((o == mine) & (q0 + j < p));
-            }
-        }
+#pragma unroll 4
+    for (int q = lane; q < S; q += 32) {
+        const long long o = F[q];
+        rank += (o > mine) | ((o == mine) & (q < p));
     }
-    if (p < S) ds.d.order[rank] = p;
+    rank = __reduce_add_sync(kFull, rank);
+    if (lane == 0) ds.d.order[rank] = p;
 }
 
 __global__ void philox_draws_kernel(unsigned long long seed, uint32_t phase, uint32_t iter,
@@ -574,14 +625,15 @@ cudaError_t launch_fitness(const int* C, int ldc, int n, const uint16_t* tours, 
 
 cudaError_t launch_det_orders(const int* tags, int n, uint16_t* orders, int ldn, int* err,
                               cudaStream_t st) {
-    dim3 grid((n + 255) / 256, 8);
+    dim3 grid((n + 31) / 32, 8);
     det_orders_kernel<<<grid, 256, 0, st>>>(tags, n, orders, ldn, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_init_particles(const Consts& k, const SwarmDev& d, const uint16_t* orders,
                                   int n_det, cudaStream_t st) {
-    init_particles_kernel<<<(k.S + 63) / 64, 64, 0, st>>>(k, d, orders, n_det);
+    const size_t smem = 2 * static_cast<size_t>(k.ldn) * sizeof(uint16_t);  // at most 32 KB
+    init_particles_kernel<<<k.S, 32, smem, st>>>(k, d, orders, n_det);
     return cudaGetLastError();
 }
 
@@ -602,24 +654,23 @@ cudaError_t launch_move(const BatchView& b, cudaStream_t st) {
 
 cudaError_t launch_mutation(const BatchView& b, cudaStream_t st) {
     if (b.total <= 0) return cudaSuccess;
-    const int wb = (b.total * 32 + 255) / 256, tb = (b.total + 255) / 256;
-    mut_hash_kernel<<<wb, 256, 0, st>>>(b);
-    mut_dup_kernel<<<tb, 256, 0, st>>>(b);
-    mut_kept_kernel<<<tb, 256, 0, st>>>(b);
+    const int wb = (b.total * 32 + 255) / 256;
+    mut_dup_kernel<<<wb, 256, 0, st>>>(b);
+    mut_kept_kernel<<<wb, 256, 0, st>>>(b);
     mut_apply_kernel<<<wb, 256, 0, st>>>(b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rank_cost(const BatchView& b, cudaStream_t st) {
-    if (b.ninst <= 0 || b.max_S <= 0) return cudaSuccess;
-    dim3 grid((b.max_S + 255) / 256, b.ninst);
-    rank_cost_kernel<<<grid, 256, 0, st>>>(b);
+    if (b.total <= 0) return cudaSuccess;
+    rank_cost_kernel<<<(b.total * 32 + 255) / 256, 256, 0, st>>>(b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gbest(const BatchView& b, int second, cudaStream_t st) {
     if (b.ninst <= 0) return cudaSuccess;
-    gbest_kernel<<<b.ninst, 1024, 0, st>>>(b, second);
+    const int threads = min(1024, max(128, round_up(b.max_S, 32)));
+    gbest_kernel<<<b.ninst, threads, 0, st>>>(b, second);
     return cudaGetLastError();
 }
 
