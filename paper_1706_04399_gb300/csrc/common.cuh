@@ -172,6 +172,7 @@ cudaError_t launch_philox_draws(unsigned long long seed, uint32_t phase, uint32_
 struct TwoOptTask {
     const int* C;
     const int* Cs;  // optional: four row-shifted copies of C (build_shifted_copies)
+    const int2* near;  // optional: neighbour lists (build_near)
     int ldc, n;
     uint16_t* tours;
     int ldt, count;
@@ -218,6 +219,13 @@ struct TwoOptBatch {
 // (short tours: two_opt_small.cu), or on the tiled kernel when a shape of it
 // is pinned (rows > 0).
 cudaError_t launch_two_opt(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+// Neighbour lists: near[kNear u + k] = {C[u][v], v} for the kNear cheapest
+// other cities v of u, in increasing order; for tours the list kernel takes.
+constexpr int kNear = 32;
+inline size_t near_bytes(int n) { return static_cast<size_t>(n) * kNear * sizeof(int2); }
+// Whether the default 2-opt launch over `total` tours of n viewpoints reads them.
+bool near_used(int n, int total, int num_sms);
+cudaError_t build_near(const int* C, int ldc, int n, int2* near, cudaStream_t st);
 // ---- two_opt_small.cu: short tours ----
 int two_opt_small_threads(int n);  // threads per tour, 0 when n is too long
 cudaError_t launch_two_opt_small(const TwoOptBatch& b, int num_sms, cudaStream_t st);

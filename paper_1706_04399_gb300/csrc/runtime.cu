@@ -87,6 +87,7 @@ struct dpso_swarm {
     SwarmDev d{};
     int* C = nullptr;
     int* Cs = nullptr;  // row-shifted copies of C for the tiled 2-opt (or null)
+    int2* near = nullptr;  // neighbour lists for the list 2-opt (or null)
     uint16_t *X = nullptr, *V = nullptr, *P = nullptr, *G = nullptr;
     long long *F = nullptr, *PF = nullptr;
     unsigned long long* hash = nullptr;
@@ -125,7 +126,7 @@ void free_swarm(dpso_swarm* s) {
     }
     for (cudaEvent_t e : s->ev_cap)
         if (e) cudaEventDestroy(e);
-    void* bufs[] = {s->C,    s->Cs,   s->X,   s->V,     s->P,   s->G,    s->F,    s->PF,
+    void* bufs[] = {s->C,    s->Cs,   s->near, s->X,   s->V,     s->P,   s->G,    s->F,    s->PF,
                     s->hash, s->dup,  s->kept, s->order, s->ctl, s->meta, s->hist};
     for (void* b : bufs)
         if (b) cudaFree(b);
@@ -152,6 +153,7 @@ TwoOptTask swarm_task(const dpso_swarm* s) {
     TwoOptTask a{};
     a.C = s->C;
     a.Cs = s->Cs;
+    a.near = s->near;
     a.ldc = s->k.ldc;
     a.n = s->k.n;
     a.tours = s->X;
@@ -430,8 +432,11 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
         TwoOptTask task;
         int toff[2];
     };
+    // followed by the 2-opt's neighbour lists
+    const size_t head = (sizeof(Scratch) + 255) / 256 * 256;
+    const bool lists = kind == 0 && near_used(n, count, sms);
     Scratch* scratch = nullptr;
-    if (cudaMallocAsync(&scratch, sizeof(Scratch), st) != cudaSuccess) {
+    if (cudaMallocAsync(&scratch, head + (lists ? near_bytes(n) : 0), st) != cudaSuccess) {
         cudaGetLastError();
         return DPSO_ERR_NO_MEMORY;
     }
@@ -452,6 +457,10 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
         e = launch_fitness(C_dev, n, n, tours_dev, n, count, reinterpret_cast<long long*>(cost_dev),
                            st);
         TwoOptTask& a = host.task;
+        if (lists) {
+            a.near = reinterpret_cast<int2*>(reinterpret_cast<char*>(scratch) + head);
+            if (e == cudaSuccess) e = build_near(C_dev, n, n, const_cast<int2*>(a.near), st);
+        }
         a.C = C_dev;
         a.ldc = n;
         a.n = n;
@@ -623,6 +632,12 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
         return fail2(DPSO_ERR_CUDA);
     if (herr & 1) return fail2(DPSO_ERR_ARG);
     if (herr & 2) return fail2(DPSO_ERR_RANGE);
+    // (alone, or with many others' tours in a batch)
+    if ((p->flags & DPSO_FLAG_TWO_OPT) && !node_swap &&
+        (near_used(n, k.S, s->num_sms) || near_used(n, 1 << 24, s->num_sms))) {
+        if ((st = dalloc(&s->near, static_cast<size_t>(n) * kNear, ust))) return fail2(st);
+        if (build_near(s->C, k.ldc, n, s->near, ust) != cudaSuccess) return fail2(DPSO_ERR_CUDA);
+    }
     {
         SwarmMeta m{};
         m.desc.k = k;

@@ -31,17 +31,27 @@
 //    to the list, the smallest delta past T' becomes the slot's low.
 //  * T' is the largest, over groups of threads, of the group's smallest low:
 //    about G ln G rows for G groups, a few scans per move in all.
+// Longer tours (kLists) also save on those scans:
+//  * Every city has a list of its 32 cheapest neighbours.  A pair that shows in
+//    neither list of an edge's two ends costs at least the lists' radii there,
+//    so where those keep its delta at or past T' the row's scan reads the two
+//    lists (a "short" row: four fifths of them) instead of all n slots.
+//  * A new edge's pair costs at least the cheapest neighbours of its two ends.
+//    A first pass over len and low picks the slots where that bound lies below
+//    T, or below the low of a longer slot; only those pairs are evaluated.
 // With T = 0 and no candidate that fits, the tour is 2-optimal.
 //
 // A list that runs full folds its upper part back into low (T falls).  Where
 // more candidates than it holds tie on one delta, so that T cannot rise, a
 // pass scans every row with low < 0 and takes the best directly.
 //
-// What bounds it: a row scan reads the cost rows of the edge's two ends from
-// L2 (staged interleaved in shared memory, so that one 8-byte gather brings
-// both ends' costs to a city) and gathers them at both ends of every other
-// edge: shared-memory gathers with random bank conflicts, then issue slots.
-// Short tours wait for L2 and barriers; several tours per SM hide that.
+// What bounds it: for long tours the gathers of the rows that are scanned in
+// full (the cost rows of the edge's two ends, staged interleaved in shared
+// memory, so that one 8-byte gather brings both ends' costs to a city) and of
+// the new edges' pairs; for short ones the issue slots and the chain of a
+// pass, about 9000 cycles at n = 400.  Against scanning every row and every
+// pair of the new edges, on GB300: 600 tours at n = 1992 39 -> 28 ms, 150 at
+// n = 2999 28 -> 19, 600 at n = 1000 10.1 -> 7.1.
 #include <climits>
 
 #include "tiled_common.cuh"
@@ -51,7 +61,7 @@ namespace {
 
 using namespace tiled;
 
-constexpr int kThreadsPerSm = 768;  // the register budget's resident threads
+constexpr int kThreadsPerSm = 640;  // the register budget's resident threads
 constexpr int kBig = 1 << 30;  // on a staged row's own city: a pair that shares it never improves
 constexpr unsigned long long kDead = ~0ull;  // a dropped list entry
 
@@ -83,20 +93,57 @@ __host__ __device__ constexpr size_t list_smem(int n, int bufs, bool full, int c
     const size_t m = (n + 7) / 8 * 8;
     const size_t staged =
         full ? (static_cast<size_t>(n) * full_ld(n) + 3) / 4 * 16 : m * bufs * sizeof(int2);
-    return staged + m * (sizeof(unsigned) + 2 * sizeof(int) + 3 * sizeof(uint16_t)) +
+    return staged + m * (2 * sizeof(unsigned) + 2 * sizeof(int) + 3 * sizeof(uint16_t)) +
            static_cast<size_t>(cap) * sizeof(unsigned long long);
+}
+
+// One warp per city: its kNear cheapest neighbours, one per lane in increasing
+// (cost, city) order.  A chunk of 32 cities that holds none cheaper than the
+// dearest so far is passed over; else it is sorted and merged by a bitonic
+// network over the lanes.
+__device__ __forceinline__ unsigned long long bitonic_step(unsigned long long v, int xor_lane,
+                                                           bool up) {
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, xor_lane);
+    const bool low_lane = (threadIdx.x & xor_lane) == 0;
+    return (v < o) == (low_lane == up) ? v : o;
+}
+
+__global__ void __launch_bounds__(128) near_kernel(const int* __restrict__ C, int ldc, int n,
+                                                   int2* __restrict__ near) {
+    const int lane = threadIdx.x & 31, u = (blockIdx.x * 128 + threadIdx.x) >> 5;
+    if (u >= n) return;
+    const int* row = C + static_cast<size_t>(u) * ldc;
+    unsigned long long kept = ~0ull;
+    for (int c0 = 0; c0 < n; c0 += 32) {
+        const int c = c0 + lane;
+        unsigned long long v =
+            c < n && c != u ? (static_cast<unsigned long long>(row[c]) << 16) | c : ~0ull;
+        if (!__any_sync(0xffffffffu, v < __shfl_sync(0xffffffffu, kept, 31))) continue;
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+            for (int j = k >> 1; j > 0; j >>= 1) v = bitonic_step(v, j, (lane & k) == 0);
+        v = min(kept, __shfl_sync(0xffffffffu, v, 31 - lane));  // the 32 smallest, bitonic
+#pragma unroll
+        for (int j = 16; j > 0; j >>= 1) v = bitonic_step(v, j, true);
+        kept = v;
+    }
+    near[u * kNear + lane] =
+        kept == ~0ull ? make_int2(INT_MAX / 2, u == 0 ? 1 : 0)
+                      : make_int2(static_cast<int>(kept >> 16), static_cast<int>(kept & 0xffff));
 }
 
 // How a launch stages cost rows and shares out the rows of a scan round.
 //   kMatrix    the whole matrix in shared memory (few tours per SM: no wait for
 //              L2 after the first); every warp scans its own rows
 //   kWarpRows  each warp stages and scans its own rows (two buffers per warp)
-//   kCtaRows2  the CTA scans one row at a time while the next one arrives
-//   kCtaRows1  the same with one buffer (the longest tours)
-enum Staging { kMatrix, kWarpRows, kCtaRows2, kCtaRows1 };
+//   kCtaRows   the CTA scans one row at a time while the next one arrives
+//   kGlobal    every warp scans its own rows from C (few tours per SM, where
+//              more threads serve a tour than could stage; the longest tours)
+enum Staging { kMatrix, kWarpRows, kCtaRows, kGlobal };
 
 __host__ __device__ constexpr int staged_bufs(int threads, Staging st) {
-    return st == kWarpRows ? 2 * (threads / 32) : (st == kCtaRows1 ? 1 : 2);
+    return st == kWarpRows ? 2 * (threads / 32) : (st == kCtaRows ? 2 : 0);
 }
 
 // NT threads solve one tour.
@@ -106,14 +153,19 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
     constexpr int kW = NT / 32;                     // warps
     constexpr int kBufs = staged_bufs(NT, ST);      // staged row pairs
     constexpr bool kFull = ST == kMatrix;
-    constexpr bool kWarpScan = ST == kMatrix || ST == kWarpRows;
+    constexpr bool kStages = ST == kWarpRows || ST == kCtaRows;
+    constexpr bool kWarpScan = ST != kCtaRows;
+    // Neighbour lists and bounds on the new edges' pairs; short tours, whose rows
+    // are read in a few steps, are faster without (n = 400, 1024 tours: a swarm's
+    // generations 8 % slower with them).
+    constexpr bool kLists = ST == kCtaRows || ST == kGlobal;
     constexpr int kBatch = 4;                       // partners a thread has in flight
     // threads per group of the choice of T' (see the head of the file)
     constexpr int kGroup = NT / 16;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned long long s_key[2][kW];  // the warps' best, by pass parity
     __shared__ int s_lo[kW], s_hi[kW];
-    __shared__ int s_item, s_cnt, s_rows, s_drop;
+    __shared__ int s_item, s_cnt, s_rows, s_wide, s_drop;
     __shared__ long long s_pf;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -126,9 +178,10 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
     unsigned* const ends = reinterpret_cast<unsigned*>(list + cap);  // u | w << 16
     int* const len = reinterpret_cast<int*>(ends + m8);              // C[u][w]
     int* const low = len + m8;
-    uint16_t* const pos = reinterpret_cast<uint16_t*>(low + m8);  // slot -> position | dir << 15
+    unsigned* const inc = reinterpret_cast<unsigned*>(low + m8);  // city -> its two slots
+    uint16_t* const pos = reinterpret_cast<uint16_t*>(inc + m8);  // slot -> position | dir << 15
     uint16_t* const at = pos + m8;                                // position -> slot | dir << 15
-    uint16_t* const rows = at + m8;                               // slots to scan
+    uint16_t* const rows = at + m8;  // slots to scan: short rows from the front, wide from the back
 
     for (;;) {
         if (tid == 0) s_item = static_cast<int>(atomicAdd(b.queue, 1u));
@@ -145,6 +198,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
         const int n = a.n;
         const int* __restrict__ const C = a.C;
         const int ldc = a.ldc;
+        const int2* __restrict__ const near = kLists ? a.near : nullptr;
         const int max_moves = a.max_moves;
         const int mld = full_ld(n);
         uint16_t* const tour = a.tours + static_cast<size_t>(p) * a.ldt;
@@ -163,15 +217,17 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
             ends[i] = u | (w << 16);
             len[i] = d;
             low[i] = -2 * d;
+            inc[u] = i | ((i == 0 ? n - 1 : i - 1) << 16);
             pos[i] = static_cast<uint16_t>(i);
             at[i] = static_cast<uint16_t>(i);
         }
         if (tid == 0) {
             s_cnt = 0;
+            s_rows = 0;
             s_drop = INT_MAX;
         }
         long long f = a.cost[p];
-        long long scans = 0;  // rows scanned
+        long long scans = 0;  // rows decided: new edges, and rows scanned
         int moves = 0, passes = 0;
         int T = INT_MIN;      // the list holds every candidate with delta < T
         int direct = 0;       // passes to take directly (ties overflow the list)
@@ -184,7 +240,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
         // Stages the cost rows of edge (u, w) interleaved into buffer k, by
         // threads t0, t0 + step, ..: one copy group.
         auto load_rows = [&](int k, int u, int w, int t0, int step) {
-            if constexpr (!kFull) {
+            if constexpr (kStages) {
                 int2* const buf = buf0 + k * m8;
                 const int* ru = C + static_cast<size_t>(u) * ldc;
                 const int* rw = C + static_cast<size_t>(w) * ldc;
@@ -199,7 +255,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
         // After the thread's copies of the row landed: its own cities' costs
         // are such that a pair sharing a city never improves.
         auto seal_rows = [&](int k, int u, int w, int t0, int step) {
-            if constexpr (!kFull) {
+            if constexpr (kStages) {
                 if (u % step == t0) buf0[k * m8 + u].x = kBig;
                 if (w % step == t0) buf0[k * m8 + w].y = kBig;
             }
@@ -207,8 +263,18 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
         // Costs of city c to the two ends (u, w) of the edge staged in buffer k.
         auto costs = [&](int k, int u, int w, int c) {
             if constexpr (kFull) return make_int2(mat[u * mld + c], mat[w * mld + c]);
-            else return buf0[k * m8 + c];
+            else if constexpr (kStages) return buf0[k * m8 + c];
+            else return make_int2(c == u ? kBig : C[static_cast<size_t>(u) * ldc + c],
+                                  c == w ? kBig : C[static_cast<size_t>(w) * ldc + c]);
         };
+        // C between two cities; a city's cheapest and dearest listed neighbour
+        // (0 without the table: no bound, no short rows).
+        auto cost = [&](int u, int w) {
+            if constexpr (kFull) return mat[u * mld + w];
+            else return C[static_cast<size_t>(u) * ldc + w];
+        };
+        auto nearest = [&](int u) { return near ? near[u * kNear].x : 0; };
+        auto farthest = [&](int u) { return near ? near[u * kNear + kNear - 1].x : 0; };
         // The key (delta, i, j) of a candidate whose reconnection fits, else ~0.
         auto key_of = [&](int d, int e, int h, int type) {
             const unsigned pe = pos[e], ph = pos[h];
@@ -296,9 +362,13 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                 // (a round raises T by at least one; far more rounds than rows
                 // would mean one tie after another: look directly)
                 if (rounds > 1000 + n) direct = max(direct, 1);
-                if (tid == 0) s_rows = 0;
+                if (tid == 0) {
+                    s_rows = 0;
+                    s_wide = 0;
+                }
                 compact(min(s_cnt, cap));
                 int mn = INT_MAX;
+#pragma unroll 4
                 for (int s = tid; s < n; s += NT) mn = min(mn, low[s]);
                 int gm = mn;
                 for (int o = 1; o < min(kGroup << level, 32); o <<= 1)
@@ -324,20 +394,27 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                 const bool dir = direct > 0;
                 if ((kGroup << level) > (kW > 1 ? 32 : 16)) hi = lo;
                 int Tn = dir ? 0 : min(0, max(hi, lo + 1));
-                for (int s0 = 0; s0 < n; s0 += NT) {
-                    const int s = s0 + tid;
-                    const bool take = s < n && low[s] < Tn;
-                    const unsigned mask = __ballot_sync(0xffffffffu, take);
-                    if (mask == 0) continue;
-                    int k = lane == 0 ? atomicAdd(&s_rows, __popc(mask)) : 0;
-                    k = __shfl_sync(0xffffffffu, k, 0) + __popc(mask & ((1u << lane) - 1));
-                    if (take) {
-                        rows[k] = static_cast<uint16_t>(s);
-                        if (!dir) low[s] = INT_MAX;
-                    }
+                // Rows to scan.  A short row's pairs all show in the neighbour
+                // lists of its two ends: a pair that is in neither costs at
+                // least the two radii, so its delta is no less than
+                // reach - 2 len.
+                auto reach = [&](unsigned ends_e, int len_e) {
+                    return min(farthest(ends_e & 0xffff), len_e) + min(farthest(ends_e >> 16), len_e);
+                };
+                unsigned take = 0;  // bit k: this thread's k-th slot (at most 32)
+#pragma unroll 4
+                for (int s = tid, k = 0; s < n; s += NT, ++k)
+                    take |= static_cast<unsigned>(low[s] < Tn) << k;
+                for (; take; take &= take - 1) {
+                    const int s = tid + (__ffs(take) - 1) * NT;
+                    const bool wide = reach(ends[s], len[s]) - 2 * len[s] < Tn;
+                    const int k = atomicAdd(wide ? &s_wide : &s_rows, 1);
+                    rows[wide ? n - 1 - k : k] = static_cast<uint16_t>(s);
+                    if (!dir) low[s] = INT_MAX;
                 }
                 __syncthreads();
-                const int nr = s_rows;  // at least the row whose low is lo
+                const int ns = s_rows, nr = s_wide;
+                const uint16_t* const wrows = rows + n - nr;  // (in whatever order)
                 unsigned long long mine = ~0ull;
                 // Scans the pairs that edge e (staged in buffer k) owns, over
                 // slots t0, t0 + step, ..: candidates in [T, Tn) go to the list,
@@ -385,58 +462,108 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                 };
                 auto load_row = [&](int k, int r, int t0, int step) {
                     if (r < nr) {
-                        const unsigned v = ends[rows[r]];
+                        const unsigned v = ends[wrows[r]];
                         load_rows(k, v & 0xffff, v >> 16, t0, step);
                     } else {
                         cp_commit();
                     }
                 };
                 auto seal_row = [&](int k, int r, int t0, int step) {
-                    const unsigned v = ends[rows[r]];
+                    const unsigned v = ends[wrows[r]];
                     seal_rows(k, v & 0xffff, v >> 16, t0, step);
+                };
+                // Scans the short rows, eight lanes for each end of an edge, four
+                // neighbours per lane: their costs are read together, then those
+                // of the pairs they leave open (two waits for L2 per row).
+                auto scan_short = [&]() {
+                    constexpr int kPer = kNear / 8;
+                    for (int i0 = 4 * warp; i0 < 2 * ns; i0 += 4 * kW) {
+                        const int item = min(i0 + (lane >> 3), 2 * ns - 1);
+                        const bool on = i0 + (lane >> 3) < 2 * ns;
+                        const int e = rows[item >> 1], side = item & 1;
+                        const unsigned ve = ends[e];
+                        const int u = side ? ve >> 16 : ve & 0xffff, w = side ? ve & 0xffff : ve >> 16;
+                        const int de = len[e];
+                        int2 nb[kPer];
+#pragma unroll
+                        for (int k = 0; k < kPer; ++k) nb[k] = near[u * kNear + (lane & 7) + 8 * k];
+                        const int rw = min(farthest(w), de);
+                        const int ru =
+                            min(__shfl_sync(0xffffffffu, nb[kPer - 1].x, (lane & 24) + 7), de);
+                        int lbe = ru + rw - 2 * de;  // what the lists leave out
+                        int c2[2 * kPer], slot[2 * kPer];
+#pragma unroll
+                        for (int k = 0; k < kPer; ++k) {
+                            const int v = nb[k].y;
+                            const bool listed = on && nb[k].x < ru && v != w;
+                            const unsigned two = inc[v];
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const int s = q ? two >> 16 : two & 0xffff, ds = len[s];
+                                const unsigned vs = ends[s];
+                                const bool first = static_cast<int>(vs & 0xffff) == v;
+                                const int z = first ? vs >> 16 : vs & 0xffff;
+                                const bool open = listed && ds <= de - (s >= e ? 1 : 0) && z != u &&
+                                                  z != w && nb[k].x - de - ds < 0;
+                                slot[2 * k + q] = open ? s | (first ? 0x2000 : 0) : -1;
+                                if (open) c2[2 * k + q] = cost(w, z);
+                            }
+                        }
+#pragma unroll
+                        for (int k = 0; k < 2 * kPer; ++k) {
+                            if (slot[k] < 0 || (side && c2[k] < rw)) continue;  // (the other end lists it)
+                            const int s = slot[k] & 0x1fff, d = nb[k / 2].x + c2[k] - de - len[s];
+                            const int type = (slot[k] >> 13) == (side == 0 ? 1 : 0) ? 0 : 1;
+                            if (d >= Tn) lbe = min(lbe, d);
+                            else if (dir) mine = min(mine, d < 0 ? key_of(d, e, s, type) : ~0ull);
+                            else if (d >= T) insert(d, e, s, type);
+                        }
+#pragma unroll
+                        for (int o = 1; o < 8; o <<= 1)
+                            lbe = min(lbe, __shfl_xor_sync(0xffffffffu, lbe, o));
+                        if (on && !dir && (lane & 7) == 0 && lbe < 0) atomicMin(&low[e], lbe);
+                    }
                 };
                 bool shrunk = false;
                 for (;;) {
-                    scans += nr;
+                    scans += nr + ns;
+                    scan_short();
                     if constexpr (kWarpScan) {
-                        if (!kFull) load_row(2 * warp, warp, lane, 32);
+                        if (kStages) load_row(2 * warp, warp, lane, 32);
                         for (int r = warp, q = 0; r < nr; r += kW, q ^= 1) {
                             const int k = 2 * warp + q;
-                            if (!kFull) {
+                            if (kStages) {
                                 load_row(2 * warp + (q ^ 1), r + kW, lane, 32);
                                 cp_wait<1>();
                                 seal_row(k, r, lane, 32);
                             }
                             __syncwarp();
-                            const int e = rows[r];
+                            const int e = wrows[r];
                             const int lbe = scan(k, e, lane, 32);
-                            if (!dir && lane == 0) low[e] = lbe;
+                            if (!dir && lane == 0) atomicMin(&low[e], lbe);
                             __syncwarp();  // the buffer is no longer read
                         }
-                        if (!kFull) cp_wait_all();
+                        if (kStages) cp_wait_all();
                     } else {
-                        load_row(0, 0, tid, NT);
+                        if (nr > 0) load_row(0, 0, tid, NT);
                         for (int r = 0; r < nr; ++r) {
-                            const int k = ST == kCtaRows2 ? r & 1 : 0;
+                            const int k = r & 1;
                             cp_wait_all();
                             seal_row(k, r, tid, NT);
                             __syncthreads();
-                            if (ST == kCtaRows2 && r + 1 < nr) load_row(k ^ 1, r + 1, tid, NT);
-                            const int e = rows[r];
+                            if (r + 1 < nr) load_row(k ^ 1, r + 1, tid, NT);
+                            const int e = wrows[r];
                             const int lbe = scan(k, e, tid, NT);
                             if (!dir && lane == 0) atomicMin(&low[e], lbe);
-                            if (ST == kCtaRows1 && r + 1 < nr) {
-                                __syncthreads();  // the buffer is no longer read
-                                load_row(0, r + 1, tid, NT);
-                            }
                         }
                     }
                     __syncthreads();
                     if (s_cnt <= cap) break;
-                    // The list ran full: T' falls to the largest, over 32
-                    // groups of threads, of the group's smallest delta, what this round added is dropped and its
-                    // rows are scanned again.  Where T' cannot stay above T
-                    // (ties), T falls too and the next passes are direct.
+                    // The list ran full: T' falls to the largest, over 32 groups of
+                    // threads, of the group's smallest delta, what this round
+                    // added is dropped and its rows are scanned again.  Where T'
+                    // cannot stay above T (ties), T falls too and the next
+                    // passes are direct.
                     int mk = INT_MAX;
                     for (int k = tid; k < cap; k += NT)
                         if (list[k] != kDead) mk = min(mk, static_cast<int>(list[k] >> 32));
@@ -481,14 +608,14 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
             const unsigned ve = ends[e], vh = ends[h];
             const int xa = ae >> 15 ? ve >> 16 : ve & 0xffff, xa1 = ae >> 15 ? ve & 0xffff : ve >> 16;
             const int xb = ah >> 15 ? vh >> 16 : vh & 0xffff, xb1 = ah >> 15 ? vh & 0xffff : vh >> 16;
-            load_rows(0, xa, xb, tid, NT);
-            if (kBufs > 1) load_rows(1, xa1, xb1, tid, NT);
-            const int cnt0 = s_cnt;
-            int de = 0, dh = 0;
-            if (tid == 0) {
-                de = kFull ? mat[xa * mld + xb] : C[static_cast<size_t>(xa) * ldc + xb];
-                dh = kFull ? mat[xa1 * mld + xb1] : C[static_cast<size_t>(xa1) * ldc + xb1];
+            if (!kLists) {
+                load_rows(0, xa, xb, tid, NT);
+                load_rows(1, xa1, xb1, tid, NT);
             }
+            const int cnt0 = s_cnt;
+            // the new edges, and the least a pair can cost at their ends
+            const int de = cost(xa, xb), dh = cost(xa1, xb1);
+            const int least_e = nearest(xa) + nearest(xb), least_h = nearest(xa1) + nearest(xb1);
             // candidates of the removed edges go
             for (int k = tid; k < cnt0; k += NT) {
                 const unsigned lo = static_cast<unsigned>(list[k]);
@@ -510,48 +637,91 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                 ends[h] = xa1 | (xb1 << 16);
                 len[e] = de;
                 len[h] = dh;
-                low[e] = INT_MAX;
-                low[h] = INT_MAX;
+                low[e] = kLists ? max(T, least_e - 2 * de) : INT_MAX;
+                low[h] = kLists ? max(T, least_h - 2 * dh) : INT_MAX;
+                // xb changes from h to e, xa1 from e to h
+                const unsigned ib = inc[xb], ia = inc[xa1];
+                inc[xb] = static_cast<int>(ib & 0xffff) == h ? (ib & 0xffff0000u) | e
+                                                             : (ib & 0xffff) | (e << 16);
+                inc[xa1] = static_cast<int>(ia & 0xffff) == e ? (ia & 0xffff0000u) | h
+                                                              : (ia & 0xffff) | (h << 16);
                 at[bi] = static_cast<uint16_t>(e);
                 at[bj] = static_cast<uint16_t>(h);
                 pos[e] = static_cast<uint16_t>(bi);
                 pos[h] = static_cast<uint16_t>(bj);
+                s_rows = 0;
             }
-            if (!kFull) cp_wait_all();
-            seal_rows(0, xa, xb, tid, NT);
-            if (kBufs > 1) seal_rows(1, xa1, xb1, tid, NT);
+            if (!kLists && !kFull) {
+                cp_wait_all();
+                seal_rows(0, xa, xb, tid, NT);
+                seal_rows(1, xa1, xb1, tid, NT);
+            }
             __syncthreads();
 
-            // The new edge x (staged in buffer k) against every other but
-            // `skip`: candidates below T go to the list, the smallest delta past
-            // T to the low of the pair's owner.
-            auto against = [&](int k, int x, int u, int w, int skip) {
-                const int dx = len[x];
-                int lbx = INT_MAX;
-                for (int s0 = tid; s0 < n; s0 += kBatch * NT) {
-                    int d0[kBatch], d1[kBatch], ml[kBatch], m = INT_MAX;
-                    bool lower = false;
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q) {
-                        const int s = min(s0 + q * NT, n - 1);
-                        const unsigned v = ends[s];
-                        const int ds = len[s];
-                        const int2 A = costs(k, u, w, v & 0xffff);
-                        const int2 B = costs(k, u, w, v >> 16);
-                        const bool ok = s0 + q * NT < n && s != x && s != skip;
-                        d0[q] = ok ? A.x + B.y - dx - ds : INT_MAX;
-                        d1[q] = ok ? B.x + A.y - dx - ds : INT_MAX;
-                        const int mq = min(d0[q], d1[q]);
-                        const bool own = ds <= dx - (s >= x ? 1 : 0);
-                        m = min(m, mq);
-                        lbx = min(lbx, own && mq >= T ? mq : INT_MAX);
-                        ml[q] = own ? INT_MAX : mq;
-                        lower = lower || ml[q] < low[s];
+            if constexpr (kLists) {
+                // The pairs of the two new edges.  Their deltas are no less than
+                // least - (both edges), so only slots where that is below T, or
+                // below the low of a longer slot, are looked at: their own lows
+                // start at that bound.
+                {
+                    unsigned fe = 0, fh = 0;  // bit k: this thread's k-th slot (at most 32)
+#pragma unroll 4
+                    for (int s = tid, k = 0; s < n; s += NT, ++k) {
+                        const int ds = len[s], over = min(max(low[s], T), 0);
+                        const bool le = least_e - de - ds < (ds > de - (s >= e ? 1 : 0) ? over : T);
+                        const bool lh = least_h - dh - ds < (ds > dh - (s >= h ? 1 : 0) ? over : T);
+                        fe |= static_cast<unsigned>(le && s != e) << k;
+                        fh |= static_cast<unsigned>(lh && s != h && s != e) << k;
                     }
-                    if (m < T || lower) {
+                    const int mine = __popc(fe | fh);
+                    int upto = mine;
 #pragma unroll
-                        for (int q = 0; q < kBatch; ++q) {
-                            const int s = s0 + q * NT;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, upto, o);
+                        if (lane >= o) upto += y;
+                    }
+                    int k = lane == 31 ? atomicAdd(&s_rows, upto) : 0;
+                    k = __shfl_sync(0xffffffffu, k, 31) + upto - mine;
+                    for (unsigned f = fe | fh; f; f &= f - 1) {
+                        const int bit = __ffs(f) - 1;
+                        rows[k++] = static_cast<uint16_t>((tid + bit * NT) | (fe >> bit & 1) << 13 |
+                                                          (fh >> bit & 1) << 14);
+                    }
+                }
+                __syncthreads();
+                {
+                    // (a thread's entries' costs are read together)
+                    constexpr int kHits = 4;
+                    const int hits = 2 * s_rows;
+                    for (int k0 = tid; k0 < hits; k0 += kHits * NT) {
+                        int d0[kHits], d1[kHits], slot[kHits];
+#pragma unroll
+                        for (int q = 0; q < kHits; ++q) {
+                            const int k = k0 + q * NT;
+                            const int v = k < hits ? rows[k >> 1] : 0, s = v & 0x1fff;
+                            const bool second = k & 1;
+                            const int u = second ? xa1 : xa, w = second ? xb1 : xb;
+                            const unsigned vs = ends[s];
+                            const int c0 = vs & 0xffff, c1 = vs >> 16;
+                            // (a shared city: one reconnection changes nothing, the
+                            // other is none)
+                            const bool on = (v & (second ? 0x4000 : 0x2000)) && c0 != u && c0 != w &&
+                                            c1 != u && c1 != w;
+                            slot[q] = on ? s : -1;
+                            if (on) {
+                                const int both = (second ? dh : de) + len[s];
+                                d0[q] = cost(u, c0) + cost(w, c1) - both;
+                                d1[q] = cost(u, c1) + cost(w, c0) - both;
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < kHits; ++q) {
+                            const int s = slot[q];
+                            if (s < 0) continue;
+                            const bool second = (k0 + q * NT) & 1;
+                            const int x = second ? h : e, dx = second ? dh : de;
+                            const int own = len[s] <= dx - (s >= x ? 1 : 0) ? x : s;
+                            if (min(d0[q], d1[q]) >= low[own]) continue;  // (T <= low)
                             int keep = INT_MAX;  // the smallest not in the list
 #pragma unroll
                             for (int type = 0; type < 2; ++type) {
@@ -562,23 +732,62 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                                 }
                                 keep = min(keep, d);
                             }
-                            if (ml[q] == INT_MAX) lbx = min(lbx, keep);
-                            else if (keep < low[s]) atomicMin(&low[s], keep);
+                            if (keep < low[own]) atomicMin(&low[own], keep);
                         }
                     }
                 }
-                lbx = __reduce_min_sync(0xffffffffu, lbx);
-                if (lane == 0) atomicMin(&low[x], lbx);
-            };
-            against(0, e, xa, xb, -1);
-            if (kBufs == 1) {
-                __syncthreads();
-                load_rows(0, xa1, xb1, tid, NT);
-                cp_wait_all();
-                seal_rows(0, xa1, xb1, tid, NT);
-                __syncthreads();
+            } else {
+                // The new edge x (staged in buffer k) against every other but
+                // `skip`: candidates below T go to the list, the smallest delta past
+                // T to the low of the pair's owner.
+                auto against = [&](int k, int x, int u, int w, int skip) {
+                    const int dx = len[x];
+                    int lbx = INT_MAX;
+                    for (int s0 = tid; s0 < n; s0 += kBatch * NT) {
+                        int d0[kBatch], d1[kBatch], ml[kBatch], m = INT_MAX;
+                        bool lower = false;
+#pragma unroll
+                        for (int q = 0; q < kBatch; ++q) {
+                            const int s = min(s0 + q * NT, n - 1);
+                            const unsigned v = ends[s];
+                            const int ds = len[s];
+                            const int2 A = costs(k, u, w, v & 0xffff);
+                            const int2 B = costs(k, u, w, v >> 16);
+                            const bool ok = s0 + q * NT < n && s != x && s != skip;
+                            d0[q] = ok ? A.x + B.y - dx - ds : INT_MAX;
+                            d1[q] = ok ? B.x + A.y - dx - ds : INT_MAX;
+                            const int mq = min(d0[q], d1[q]);
+                            const bool own = ds <= dx - (s >= x ? 1 : 0);
+                            m = min(m, mq);
+                            lbx = min(lbx, own && mq >= T ? mq : INT_MAX);
+                            ml[q] = own ? INT_MAX : mq;
+                            lower = lower || ml[q] < low[s];
+                        }
+                        if (m < T || lower) {
+#pragma unroll
+                            for (int q = 0; q < kBatch; ++q) {
+                                const int s = s0 + q * NT;
+                                int keep = INT_MAX;  // the smallest not in the list
+#pragma unroll
+                                for (int type = 0; type < 2; ++type) {
+                                    const int d = type ? d1[q] : d0[q];
+                                    if (d < T) {
+                                        if (insert(d, x, s, type)) continue;
+                                        atomicMin(&s_drop, d);  // T falls to it after the pass
+                                    }
+                                    keep = min(keep, d);
+                                }
+                                if (ml[q] == INT_MAX) lbx = min(lbx, keep);
+                                else if (keep < low[s]) atomicMin(&low[s], keep);
+                            }
+                        }
+                    }
+                    lbx = __reduce_min_sync(0xffffffffu, lbx);
+                    if (lane == 0) atomicMin(&low[x], lbx);
+                };
+                against(0, e, xa, xb, -1);
+                against(1, h, xa1, xb1, e);
             }
-            against(kBufs > 1 ? 1 : 0, h, xa1, xb1, e);
             scans += 2;
             ++moves;
             __syncthreads();
@@ -642,20 +851,18 @@ cudaError_t launch_cfg(const TwoOptBatch& b, int cap, int num_sms, cudaStream_t 
 
 // Launch configurations: for tours of up to max_n viewpoints (and, with
 // `few`, launches of at most that many tours per SM): threads per tour,
-// staging, list entries.  Measured on GB300 (random grid and facade tours to
-// 2-optimality, us; calls of one move taken off up to n = 220):
-//   n     tours  matrix, 256 thr.  warp rows, 64 thr.  warp rows, 128 thr.
-//   90    32     178               305                 256
-//   90    1024   578               483                 559
-//   157   256    389               719                 529
-//   157   1024   1307              884                 1112
-//   220   128    496               980                 691
-//   220   304    907               1013                767
-//   400   256    -                 2815                2116
-//   400   1024   -                 4080                4550
-// and with the CTA's rows: n = 1000, 600 tours 10.1 ms with 128 threads, 13.9
-// with 256; n = 1992, 600 tours 45 and 39; n = 2999, 150 tours 35 and 28, 512
-// threads 29.
+// staging, list entries.  Measured on GB300 (random grid, facade and bridge
+// tours to 2-optimality, whole call, ms; warp = each warp stages its rows):
+//   n     tours  matrix 256  warp 64 / 128  CTA 128 / 256 / 512   C 128 / 256
+//   157   256    0.70        1.02 / 0.80                          0.80 / -
+//   157   1024   1.31        1.25 / 1.43                          1.39 / -
+//   220   128    0.86        -    / 1.07                          1.03 / 0.87
+//   400   256    -           3.13 / 2.30    2.45 / - / -          2.30 / 1.94
+//   400   1024   -           4.12 / 4.65    4.86 / - / -          4.60 / -
+//   1000  150    -           -              5.53 / 4.75 / -       5.67 / 4.15
+//   1000  600    -           -              7.14 / 10.0 / -       7.45 / 9.21
+//   1992  600    -           -              31.1 / 27.6 / 41.7    57.5 / 30.6
+//   2999  150    -           -              -    / 19.4 / 19.3    -    / 24.1
 struct ListConfig {
     int max_n, few, threads;
     Staging staging;
@@ -664,9 +871,10 @@ struct ListConfig {
 constexpr int kAny = INT_MAX;
 constexpr ListConfig kConfigs[] = {
     {160, 2, 256, kMatrix, 512},        {220, 1, 256, kMatrix, 512},
-    {512, 3, 128, kWarpRows, 512},      {512, kAny, 64, kWarpRows, 512},
-    {1200, kAny, 128, kCtaRows2, 1024}, {5000, kAny, 256, kCtaRows2, 1024},
-    {DPSO_MAX_N, kAny, 512, kCtaRows1, 1024},
+    {512, 2, 256, kGlobal, 512},        {512, 4, 128, kWarpRows, 512},
+    {512, kAny, 64, kWarpRows, 512},    {1200, 1, 256, kGlobal, 1024},
+    {1200, kAny, 128, kCtaRows, 1024},  {5000, kAny, 256, kCtaRows, 1024},
+    {DPSO_MAX_N, kAny, 512, kGlobal, 1024},
 };
 constexpr int kNumConfigs = sizeof(kConfigs) / sizeof(kConfigs[0]);
 
@@ -713,6 +921,17 @@ int two_opt_class(int n, int* ctas) {
     *ctas = min(static_cast<int>((228 * 1024) / (config_smem(c, n) + 1280)),
                 kThreadsPerSm / c.threads);
     return k;
+}
+
+bool near_used(int n, int total, int num_sms) {
+    if (takes_small(n, total, num_sms)) return false;
+    const Staging st = kConfigs[find_config(n, total, num_sms)].staging;
+    return st == kCtaRows || st == kGlobal;
+}
+
+cudaError_t build_near(const int* C, int ldc, int n, int2* near, cudaStream_t st) {
+    near_kernel<<<(n + 3) / 4, 128, 0, st>>>(C, ldc, n, near);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_two_opt(const TwoOptBatch& b, int num_sms, cudaStream_t st) {

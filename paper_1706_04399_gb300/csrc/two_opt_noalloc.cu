@@ -121,6 +121,14 @@ extern "C" int dpso_two_opt_noalloc(const int32_t* C_dev, int32_t n, uint16_t* t
     a.status = err;
     a.tour_passes = scratch + kHeaderWords;
     a.tour_moves = scratch + kHeaderWords + count;
+    // neighbour lists in what the counts leave of the array, when they fit
+    // (without them the kernel scans whole rows)
+    const size_t lists_at = (used + 15) / 16 * 16;
+    if (near_used(n, count, sms) && lists_at + near_bytes(n) <= kScratchBytes) {
+        int2* near = reinterpret_cast<int2*>(reinterpret_cast<char*>(scratch) + lists_at);
+        if (e == cudaSuccess) e = build_near(C_dev, n, n, near, st);
+        a.near = near;
+    }
     TwoOptTask* task = reinterpret_cast<TwoOptTask*>(scratch + kTaskWord);
     int* toff = reinterpret_cast<int*>(scratch + kOffWord);
     const int host_off[2] = {0, count};

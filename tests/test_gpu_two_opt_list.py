@@ -31,7 +31,8 @@ def _check(C_np, tours, max_moves=0, fn=None, sample=None):
 @pytest.mark.parametrize("n,count,moves", [
     (7, 9, 0), (44, 5, 0), (46, 5, 0), (64, 5, 0), (65, 480, 4), (66, 480, 4), (66, 5, 0),
     (90, 5, 0), (91, 5, 0), (160, 4, 0), (160, 470, 6), (161, 4, 0), (220, 4, 0), (221, 160, 6),
-    (221, 3, 0), (511, 3, 40), (512, 480, 2), (513, 2, 40), (1200, 2, 12), (1201, 2, 12), (5000, 1, 3), (5001, 1, 3)])
+    (221, 3, 0), (511, 3, 40), (512, 480, 2), (512, 620, 1), (513, 160, 2), (513, 2, 40),
+    (1200, 160, 1), (1200, 2, 12), (1201, 2, 12), (5000, 1, 3), (5001, 1, 3)])
 def test_launch_configurations(n, count, moves):
     C_np = inputs.random_cost_matrix(n, 31 * n, hi=1_000_000)
     _check(C_np, inputs.random_tours(n, count, 5 * n), moves)
