@@ -32,6 +32,7 @@ SOURCES = {
     "two_opt_tiled.cu": [],
     "node_swap.cu": [],
     "runtime.cu": [],
+    "scratch.cu": [],
     "two_opt_noalloc.cu": [],
     "probe.cu": [],
     "server.cu": [],

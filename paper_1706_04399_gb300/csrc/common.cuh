@@ -161,7 +161,9 @@ cudaError_t launch_gbest_init(const Consts& k, const SwarmDev& d, cudaStream_t s
 cudaError_t launch_move(const BatchView& b, cudaStream_t st);
 cudaError_t launch_mutation(const BatchView& b, cudaStream_t st);
 cudaError_t launch_rank_cost(const BatchView& b, cudaStream_t st);
-cudaError_t launch_gbest(const BatchView& b, int second, cudaStream_t st);
+// Pass 0 also zeroes the `queues` work queues of the exchange launches after it.
+cudaError_t launch_gbest(const BatchView& b, int second, unsigned int* queue, int queues,
+                         cudaStream_t st);
 cudaError_t launch_philox_draws(unsigned long long seed, uint32_t phase, uint32_t iter,
                                 uint32_t particle, int count, uint32_t* out, cudaStream_t st);
 
@@ -282,6 +284,25 @@ int two_opt_list_class(int n, int* ctas);
 bool node_swap_fits(int n);
 int node_swap_class(int n);  // launch configuration: members that agree share a launch
 cudaError_t launch_node_swap(const TwoOptBatch& b, int num_sms, cudaStream_t st);
+
+// ---- scratch.cu ----
+constexpr size_t kScratchSlotBytes = 128 * 1024;
+// Device scratch of one synchronous call.  The call waits for its stream
+// before it releases the scratch (the destructor does on every path).
+struct Scratch {
+    void* p = nullptr;
+    cudaStream_t stream = nullptr;
+    int device = 0, slot = -1;
+    cudaError_t acquire(size_t bytes, cudaStream_t st);
+    void release();
+    Scratch() = default;
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    ~Scratch() {
+        if (p) cudaStreamSynchronize(stream);
+        release();
+    }
+};
 
 // ---- runtime.cu ----
 __global__ void tours_valid_kernel(const uint16_t* tours, int n, int* err);

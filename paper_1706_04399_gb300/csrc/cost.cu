@@ -278,17 +278,18 @@ extern "C" int dpso_cost_matrix(const double* xyz_dev, int32_t n, const double* 
         cp->reserved != 0)
         return DPSO_ERR_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int* err = nullptr;
-    if (cudaMallocAsync(&err, sizeof(int), st) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
+    Scratch scratch;
+    if (scratch.acquire(sizeof(int), st) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
+    int* err = static_cast<int*>(scratch.p);
     int herr = 0;
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e == cudaSuccess)
         e = launch_cost_matrix(xyz_dev, n, boxes_dev, m, cp->uav_radius_m, cp->blocked_penalty_mm,
                                C_dev, n, err, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(err, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return DPSO_ERR_CUDA;
+    scratch.release();  // (the stream was waited for)
     if (herr & 1) return DPSO_ERR_ARG;
     if (herr & 2) return DPSO_ERR_RANGE;
     return DPSO_OK;

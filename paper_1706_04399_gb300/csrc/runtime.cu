@@ -85,8 +85,8 @@ struct dpso_swarm {
     dpso_params prm{};
     Consts k{};
     SwarmDev d{};
+    void* arena = nullptr;  // one allocation for the arrays below
     int* C = nullptr;
-    int* Cs = nullptr;  // row-shifted copies of C for the tiled 2-opt (or null)
     int2* near = nullptr;  // neighbour lists for the list 2-opt (or null)
     uint16_t *X = nullptr, *V = nullptr, *P = nullptr, *G = nullptr;
     long long *F = nullptr, *PF = nullptr;
@@ -95,17 +95,19 @@ struct dpso_swarm {
     int* order = nullptr;  // exchange order, recomputed every generation
     Ctl* ctl = nullptr;
     SwarmMeta* meta = nullptr;  // device: descriptors of this swarm as a batch of one
+    int* Cs = nullptr;  // row-shifted copies of C for the tiled 2-opt (or null)
     long long* hist = nullptr;
     int hist_cap = 0;
     int n_det = 0;
     int t_host = 0;
     cudaStream_t last = nullptr;
     cudaStream_t cap = nullptr;
-    // the two generation graphs (index 0: without mutation, 1: with it); each
-    // holds kPhaseEvents event-record nodes at the phase boundaries, which
-    // record into ev_cap unless timing mode rebinds them to pool events
-    cudaGraph_t graph[2] = {nullptr, nullptr};
+    // the generation graphs (index 0: without mutation, 1: with it), and for
+    // timing mode the same with kPhaseEvents event-record nodes at the phase
+    // boundaries, rebound to pool events before every replay
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
+    cudaGraph_t timed_graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t timed_exec[2] = {nullptr, nullptr};
     cudaGraphNode_t ev_node[2][kPhaseEvents] = {};
     cudaEvent_t ev_cap[kPhaseEvents] = {};
     // timing mode
@@ -122,12 +124,12 @@ void free_swarm(dpso_swarm* s) {
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
     for (int k = 0; k < 2; ++k) {
         if (s->exec[k]) cudaGraphExecDestroy(s->exec[k]);
-        if (s->graph[k]) cudaGraphDestroy(s->graph[k]);
+        if (s->timed_exec[k]) cudaGraphExecDestroy(s->timed_exec[k]);
+        if (s->timed_graph[k]) cudaGraphDestroy(s->timed_graph[k]);
     }
     for (cudaEvent_t e : s->ev_cap)
         if (e) cudaEventDestroy(e);
-    void* bufs[] = {s->C,    s->Cs,   s->near, s->X,   s->V,     s->P,   s->G,    s->F,    s->PF,
-                    s->hash, s->dup,  s->kept, s->order, s->ctl, s->meta, s->hist};
+    void* bufs[] = {s->arena, s->Cs, s->hist};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (s->cap) cudaStreamDestroy(s->cap);
@@ -204,14 +206,13 @@ cudaError_t enqueue_generation(dpso_swarm* s, bool mut_iter, cudaStream_t st,
     if (e == cudaSuccess) e = mark(1);
     if (e == cudaSuccess && mut_iter) e = launch_mutation(bv, st);
     if (e == cudaSuccess) e = mark(2);
-    if (e == cudaSuccess) e = launch_gbest(bv, 0, st);
+    if (e == cudaSuccess) e = launch_gbest(bv, 0, tb.queue, two ? 1 : 0, st);
     if (e == cudaSuccess) e = mark(3);
     // (with a tour per SM at most all start at once, in whatever order)
     if (e == cudaSuccess && two && s->k.S > s->num_sms) e = launch_rank_cost(bv, st);
-    if (e == cudaSuccess && two) e = cudaMemsetAsync(tb.queue, 0, sizeof(unsigned int), st);
     if (e == cudaSuccess && two) e = launch_two_opt(tb, s->num_sms, st);
     if (e == cudaSuccess) e = mark(4);
-    if (e == cudaSuccess && two) e = launch_gbest(bv, 1, st);
+    if (e == cudaSuccess && two) e = launch_gbest(bv, 1, nullptr, 0, st);
     if (e == cudaSuccess) e = mark(5);
     return e;
 }
@@ -230,10 +231,10 @@ cudaError_t launch_generation_timed(dpso_swarm* s, bool mut_iter, cudaStream_t s
     const int g = mut_iter ? 1 : 0;
     for (int q = 0; q < kPhaseEvents; ++q) {
         cudaError_t r =
-            cudaGraphExecEventRecordNodeSetEvent(s->exec[g], s->ev_node[g][q], s->ev_pool[base + q]);
+            cudaGraphExecEventRecordNodeSetEvent(s->timed_exec[g], s->ev_node[g][q], s->ev_pool[base + q]);
         if (r != cudaSuccess) return r;
     }
-    cudaError_t e = cudaGraphLaunch(s->exec[g], st);
+    cudaError_t e = cudaGraphLaunch(s->timed_exec[g], st);
     if (e == cudaSuccess) s->pending.push_back({static_cast<int>(base), g});
     return e;
 }
@@ -258,21 +259,26 @@ int collect_timing(dpso_swarm* s) {
     return DPSO_OK;
 }
 
-// Captures the generation graph with (g = 1) or without (g = 0) mutation,
-// keeps it (its event-record nodes are rebound in timing mode) and
-// instantiates it.
-int capture(dpso_swarm* s, int g) {
-    for (cudaEvent_t& e : s->ev_cap)
-        if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+// Captures the generation graph with (g = 1) or without (g = 0) mutation and
+// instantiates it; `timed`: with event-record nodes, kept to be rebound.
+int capture(dpso_swarm* s, int g, bool timed) {
+    if (timed)
+        for (cudaEvent_t& e : s->ev_cap)
+            if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(s->cap, cudaStreamCaptureModeRelaxed));
-    const cudaError_t e = enqueue_generation(s, g == 1, s->cap, s->ev_cap);
+    const cudaError_t e = enqueue_generation(s, g == 1, s->cap, timed ? s->ev_cap : nullptr);
     const cudaError_t e2 = cudaStreamEndCapture(s->cap, &graph);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
         return DPSO_ERR_CUDA;
     }
-    s->graph[g] = graph;
+    if (!timed) {
+        const cudaError_t e3 = cudaGraphInstantiate(&s->exec[g], graph, 0);
+        cudaGraphDestroy(graph);
+        return e3 == cudaSuccess ? DPSO_OK : DPSO_ERR_CUDA;
+    }
+    s->timed_graph[g] = graph;
     size_t count = 0;
     CK(cudaGraphGetNodes(graph, nullptr, &count));
     std::vector<cudaGraphNode_t> nodes(count);
@@ -291,7 +297,7 @@ int capture(dpso_swarm* s, int g) {
             }
     }
     if (found != kPhaseEvents) return DPSO_ERR_INTERNAL;
-    CK(cudaGraphInstantiate(&s->exec[g], graph, 0));
+    CK(cudaGraphInstantiate(&s->timed_exec[g], graph, 0));
     return DPSO_OK;
 }
 
@@ -425,7 +431,7 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // scratch: error word, work queue, counters, and the one-problem task list
-    struct Scratch {
+    struct Head {
         int err;
         unsigned int queue;
         unsigned long long pairs, moves;
@@ -433,19 +439,18 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
         int toff[2];
     };
     // followed by the 2-opt's neighbour lists
-    const size_t head = (sizeof(Scratch) + 255) / 256 * 256;
+    const size_t head = (sizeof(Head) + 255) / 256 * 256;
     const bool lists = kind == 0 && near_used(n, count, sms);
-    Scratch* scratch = nullptr;
-    if (cudaMallocAsync(&scratch, head + (lists ? near_bytes(n) : 0), st) != cudaSuccess) {
-        cudaGetLastError();
+    Scratch room;
+    if (room.acquire(head + (lists ? near_bytes(n) : 0), st) != cudaSuccess)
         return DPSO_ERR_NO_MEMORY;
-    }
+    Head* const scratch = static_cast<Head*>(room.p);
     int* err = &scratch->err;
     int herr = 0;
     unsigned long long counters[2] = {0, 0};
-    Scratch host{};
+    Head host{};
     host.toff[1] = count;
-    cudaError_t e = cudaMemcpyAsync(scratch, &host, sizeof(Scratch), cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaMemcpyAsync(scratch, &host, sizeof(Head), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = launch_check_cost_limit(C_dev, n, n, kind ? DPSO_NODE_SWAP_COST_MAX : DPSO_COST_MAX, err, st);
     if (e == cudaSuccess) {
         tours_valid_kernel<<<count, 256, n, st>>>(tours_dev, n, err);
@@ -485,10 +490,9 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
         if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host.task is read by the copy
     }
-    cudaFreeAsync(scratch, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaErrorMemoryAllocation) return DPSO_ERR_NO_MEMORY;
     if (e != cudaSuccess) return DPSO_ERR_CUDA;
+    room.release();  // (the stream was waited for)
     if (herr == DPSO_ERR_INTERNAL || herr == DPSO_ERR_TIMEOUT) return herr;
     if (herr & 1) return DPSO_ERR_ARG;
     if (herr & 2) return DPSO_ERR_RANGE;
@@ -577,67 +581,75 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
     k.seed = seed;
     const size_t S = static_cast<size_t>(k.S), ldn = static_cast<size_t>(k.ldn);
 
-    if ((st = dalloc(&s->C, static_cast<size_t>(n) * k.ldc, ust)) ||
-        (st = dalloc(&s->X, S * ldn, ust)) || (st = dalloc(&s->V, S * ldn, ust)) ||
-        (st = dalloc(&s->P, S * ldn, ust)) || (st = dalloc(&s->G, ldn, ust)) ||
-        (st = dalloc(&s->F, S, ust)) || (st = dalloc(&s->PF, S, ust)) ||
-        (st = dalloc(&s->hash, S, ust)) || (st = dalloc(&s->dup, S, ust)) ||
-        (st = dalloc(&s->kept, S, ust)) || (st = dalloc(&s->order, S, ust)) ||
-        (st = dalloc(&s->ctl, 1, ust)) ||
-        (st = dalloc(&s->meta, 1, ust)))
-        return fail(st);
+    // one zero-filled allocation; every array starts on 256 bytes
+    // (lists for this swarm alone, or with many others' tours in a batch)
+    const bool lists = (p->flags & DPSO_FLAG_TWO_OPT) && !node_swap &&
+                       (near_used(n, k.S, s->num_sms) || near_used(n, 1 << 24, s->num_sms));
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+        const size_t here = at;
+        at += (bytes + 255) / 256 * 256;
+        return here;
+    };
+    const size_t oC = place(sizeof(int) * n * k.ldc), oX = place(2 * S * ldn),
+                 oV = place(2 * S * ldn), oP = place(2 * S * ldn), oG = place(2 * ldn),
+                 oF = place(8 * S), oPF = place(8 * S), oHash = place(8 * S), oDup = place(S),
+                 oKept = place(S), oOrder = place(4 * S), oCtl = place(sizeof(Ctl)),
+                 oMeta = place(sizeof(SwarmMeta)), oNear = place(lists ? near_bytes(n) : 0);
+    {
+        unsigned char* base = nullptr;
+        if ((st = dalloc(&base, at, ust))) return fail(st);
+        s->arena = base;
+        s->C = reinterpret_cast<int*>(base + oC);
+        s->X = reinterpret_cast<uint16_t*>(base + oX);
+        s->V = reinterpret_cast<uint16_t*>(base + oV);
+        s->P = reinterpret_cast<uint16_t*>(base + oP);
+        s->G = reinterpret_cast<uint16_t*>(base + oG);
+        s->F = reinterpret_cast<long long*>(base + oF);
+        s->PF = reinterpret_cast<long long*>(base + oPF);
+        s->hash = reinterpret_cast<unsigned long long*>(base + oHash);
+        s->dup = base + oDup;
+        s->kept = base + oKept;
+        s->order = reinterpret_cast<int*>(base + oOrder);
+        s->ctl = reinterpret_cast<Ctl*>(base + oCtl);
+        s->meta = reinterpret_cast<SwarmMeta*>(base + oMeta);
+        if (lists) s->near = reinterpret_cast<int2*>(base + oNear);
+    }
     if ((st = ensure_history(s, 1024))) return fail(st);
     s->d = SwarmDev{s->C,    s->X,   s->V,    s->P,   s->G,    s->F,
                     s->PF,   s->hash, s->dup, s->kept, s->ctl, s->order};
-    {
-        // identity until the first generation ranks the particles
-        std::vector<int> ident(S);
-        for (size_t i = 0; i < S; ++i) ident[i] = static_cast<int>(i);
-        if (cudaMemcpyAsync(s->order, ident.data(), sizeof(int) * S, cudaMemcpyHostToDevice,
-                            ust) != cudaSuccess ||
-            cudaStreamSynchronize(ust) != cudaSuccess)
-            return fail(DPSO_ERR_CUDA);
-    }
-
-    int* err = nullptr;
-    uint16_t* orders = nullptr;
-    int* tags_dev = nullptr;
-    if ((st = dalloc(&err, 1, ust))) return fail(st);
-    auto fail2 = [&](int code) {
-        cudaFree(err);
-        cudaFree(orders);
-        cudaFree(tags_dev);
-        return fail(code);
-    };
+    // error word, back-and-forth orders and tags: scratch of this call
+    const size_t orders_at = 256, tags_at = orders_at + 2 * 8 * ldn;
+    Scratch scratch;
+    if (scratch.acquire(tags_at + (det ? sizeof(int) * 3 * n : 0), ust) != cudaSuccess)
+        return fail(DPSO_ERR_NO_MEMORY);
+    unsigned char* const tmp = static_cast<unsigned char*>(scratch.p);
+    int* const err = reinterpret_cast<int*>(tmp);
+    uint16_t* const orders = reinterpret_cast<uint16_t*>(tmp + orders_at);
+    int* const tags_dev = reinterpret_cast<int*>(tmp + tags_at);
+    if (cudaMemsetAsync(tmp, 0, tags_at, ust) != cudaSuccess) return fail(DPSO_ERR_CUDA);
     if (cudaMemcpy2DAsync(s->C, sizeof(int) * k.ldc, C_dev, sizeof(int) * n, sizeof(int) * n, n,
                           cudaMemcpyDeviceToDevice, ust) != cudaSuccess ||
         launch_check_cost_limit(s->C, n, k.ldc,
                                 node_swap ? DPSO_NODE_SWAP_COST_MAX : DPSO_COST_MAX, err,
                                 ust) != cudaSuccess)
-        return fail2(DPSO_ERR_CUDA);
+        return fail(DPSO_ERR_CUDA);
     if (det) {
         s->n_det = static_cast<int>((static_cast<long long>(k.S) * p->det_frac_pct) / 100);
         s->n_det = std::min(k.S, std::max(1, s->n_det));
-        if ((st = dalloc(&orders, 8 * ldn, ust)) ||
-            (st = dalloc(&tags_dev, 3 * static_cast<size_t>(n), ust)))
-            return fail2(st);
         if (cudaMemcpyAsync(tags_dev, tags_host, sizeof(int) * 3 * n, cudaMemcpyHostToDevice, ust) !=
                 cudaSuccess ||
             launch_det_orders(tags_dev, n, orders, k.ldn, err, ust) != cudaSuccess)
-            return fail2(DPSO_ERR_CUDA);
+            return fail(DPSO_ERR_CUDA);
     }
     int herr = 0;
     if (cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ust) != cudaSuccess ||
         cudaStreamSynchronize(ust) != cudaSuccess)
-        return fail2(DPSO_ERR_CUDA);
-    if (herr & 1) return fail2(DPSO_ERR_ARG);
-    if (herr & 2) return fail2(DPSO_ERR_RANGE);
-    // (alone, or with many others' tours in a batch)
-    if ((p->flags & DPSO_FLAG_TWO_OPT) && !node_swap &&
-        (near_used(n, k.S, s->num_sms) || near_used(n, 1 << 24, s->num_sms))) {
-        if ((st = dalloc(&s->near, static_cast<size_t>(n) * kNear, ust))) return fail2(st);
-        if (build_near(s->C, k.ldc, n, s->near, ust) != cudaSuccess) return fail2(DPSO_ERR_CUDA);
-    }
+        return fail(DPSO_ERR_CUDA);
+    if (herr & 1) return fail(DPSO_ERR_ARG);
+    if (herr & 2) return fail(DPSO_ERR_RANGE);
+    if (lists && build_near(s->C, k.ldc, n, s->near, ust) != cudaSuccess)
+        return fail(DPSO_ERR_CUDA);
     {
         SwarmMeta m{};
         m.desc.k = k;
@@ -645,9 +657,8 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
         m.task = swarm_task(s);
         m.off[1] = k.S;
         m.toff[1] = k.S;
-        if (cudaMemcpyAsync(s->meta, &m, sizeof(m), cudaMemcpyHostToDevice, ust) != cudaSuccess ||
-            cudaStreamSynchronize(ust) != cudaSuccess)
-            return fail2(DPSO_ERR_CUDA);
+        if (cudaMemcpyAsync(s->meta, &m, sizeof(m), cudaMemcpyHostToDevice, ust) != cudaSuccess)
+            return fail(DPSO_ERR_CUDA);
     }
 
     if (launch_init_particles(k, s->d, orders, s->n_det, ust) != cudaSuccess ||
@@ -658,14 +669,13 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
         cudaMemcpyAsync(&s->ctl->n_det, &s->n_det, sizeof(int), cudaMemcpyHostToDevice, ust) !=
             cudaSuccess ||
         cudaStreamSynchronize(ust) != cudaSuccess)
-        return fail2(DPSO_ERR_CUDA);
-    cudaFree(err);
-    cudaFree(orders);
-    cudaFree(tags_dev);
+        return fail(DPSO_ERR_CUDA);
+    scratch.release();
 
     if (cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) != cudaSuccess)
         return fail(DPSO_ERR_CUDA);
-    if ((st = capture(s, 0)) || (st = capture(s, 1))) return fail(st);
+    if ((st = capture(s, 0, false))) return fail(st);
+    if ((k.flags & DPSO_FLAG_MUTATION) && (st = capture(s, 1, false))) return fail(st);
     *out = s;
     return DPSO_OK;
 }
@@ -843,6 +853,11 @@ int dpso_set_timing(dpso_swarm* s, int on) {
     CK(cudaStreamSynchronize(s->last));
     s->pending.clear();
     s->acc = dpso_timing{};
+    for (int g = 0; on && g < 2; ++g) {  // the graphs with event nodes, once
+        if (s->timed_exec[g] || (g == 1 && !(s->k.flags & DPSO_FLAG_MUTATION))) continue;
+        const int st = capture(s, g, true);
+        if (st) return st;
+    }
     s->timing = on != 0;
     return DPSO_OK;
 }
@@ -873,7 +888,6 @@ struct dpso_batch {
     struct TwoOptClass {
         TwoOptTask* tasks = nullptr;  // device, the class's members by descending n
         int* toff = nullptr;          // device, tour offsets (nprob + 1)
-        unsigned int* queue = nullptr;
         TwoOptBatch tb{};
     };
     int device = 0, num_sms = 0;
@@ -885,6 +899,7 @@ struct dpso_batch {
     std::vector<TwoOptTask> tasks;       // host: every exchanging member, by descending n
     std::vector<dpso_swarm*> owners;     // the members the tasks belong to
     std::vector<TwoOptClass> cls;
+    unsigned int* queues = nullptr;      // device: a work queue per class
     std::vector<cudaStream_t> side;      // capture streams of the classes after the first
     std::vector<cudaEvent_t> ev;         // fork, then one join per side stream
     cudaStream_t cap = nullptr;
@@ -896,11 +911,13 @@ namespace {
 
 void free_classes(dpso_batch* b) {
     for (auto& c : b->cls) {
-        void* bufs[] = {c.tasks, c.toff, c.queue};
+        void* bufs[] = {c.tasks, c.toff};
         for (void* p : bufs)
             if (p) cudaFree(p);
     }
     b->cls.clear();
+    if (b->queues) cudaFree(b->queues);
+    b->queues = nullptr;
 }
 
 void free_batch(dpso_batch* b) {
@@ -968,6 +985,10 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
             runs.back().second = i + 1;
         }
     }
+    if (!runs.empty()) {
+        const int st = dalloc(&b->queues, runs.size(), b->last);
+        if (st) return st;
+    }
     for (size_t c = 0; c < runs.size(); ++c) {
         dpso_batch::TwoOptClass cl;
         const int first = runs[c].first, cnt = runs[c].second - runs[c].first;
@@ -980,8 +1001,7 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
             shifted = shifted && b->tasks[i].Cs != nullptr;
         }
         int st = DPSO_OK;
-        if ((st = dalloc(&cl.tasks, cnt, b->last)) || (st = dalloc(&cl.toff, cnt + 1, b->last)) ||
-            (st = dalloc(&cl.queue, 1, b->last))) {
+        if ((st = dalloc(&cl.tasks, cnt, b->last)) || (st = dalloc(&cl.toff, cnt + 1, b->last))) {
             b->cls.push_back(cl);
             return st;
         }
@@ -992,7 +1012,7 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
                            b->last));
         CK(cudaStreamSynchronize(b->last));  // the host vectors go out of scope
         TwoOptBatch& tb = b->cls.back().tb;
-        tb = TwoOptBatch{cl.tasks, cl.toff, cnt, toff.back(), max_n, shifted, 0, cl.queue};
+        tb = TwoOptBatch{cl.tasks, cl.toff, cnt, toff.back(), max_n, shifted, 0, b->queues + c};
         tb.kind = keys[c].kind;
         if (keys[c].kind == 1) {
             // node swap: the launch follows max_n
@@ -1022,24 +1042,23 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
 cudaError_t enqueue_batch_classes(dpso_batch* b, cudaStream_t st) {
     cudaError_t e = launch_move(b->bv, st);
     if (e == cudaSuccess) e = launch_mutation(b->bv, st);
-    if (e == cudaSuccess) e = launch_gbest(b->bv, 0, st);
+    if (e == cudaSuccess)
+        e = launch_gbest(b->bv, 0, b->queues, static_cast<int>(b->cls.size()), st);
     if (e != cudaSuccess || !b->any_two_opt) return e;
     if (b->bv.total > b->num_sms) e = launch_rank_cost(b->bv, st);
     if (e == cudaSuccess && b->cls.size() > 1) e = cudaEventRecord(b->ev[0], st);
     for (size_t c = 1; c < b->cls.size() && e == cudaSuccess; ++c) {
         cudaStream_t s = b->side[c - 1];
         e = cudaStreamWaitEvent(s, b->ev[0], 0);
-        if (e == cudaSuccess) e = cudaMemsetAsync(b->cls[c].queue, 0, sizeof(unsigned int), s);
         if (e == cudaSuccess) e = launch_two_opt(b->cls[c].tb, b->num_sms, s);
         if (e == cudaSuccess) e = cudaEventRecord(b->ev[c], s);
     }
     if (e == cudaSuccess && !b->cls.empty()) {
-        e = cudaMemsetAsync(b->cls[0].queue, 0, sizeof(unsigned int), st);
-        if (e == cudaSuccess) e = launch_two_opt(b->cls[0].tb, b->num_sms, st);
+        e = launch_two_opt(b->cls[0].tb, b->num_sms, st);
     }
     for (size_t c = 1; c < b->cls.size() && e == cudaSuccess; ++c)
         e = cudaStreamWaitEvent(st, b->ev[c], 0);
-    if (e == cudaSuccess) e = launch_gbest(b->bv, 1, st);
+    if (e == cudaSuccess) e = launch_gbest(b->bv, 1, nullptr, 0, st);
     return e;
 }
 

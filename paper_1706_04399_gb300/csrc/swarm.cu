@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(32) init_particles_kernel(Consts k, SwarmDev d
     uint16_t* v = d.V + (size_t)p * k.ldn;
     uint16_t* y = sm;            // the permutation
     uint16_t* with = sm + k.ldn;  // swap partner of position i
+    if (lane == 0) d.order[p] = p;  // until the first generation ranks the particles
     if (p < n_det) {
         const uint16_t* ord = orders + (size_t)(p % 8) * k.ldn;
         const int rot = (p / 8) % n;
@@ -537,7 +538,9 @@ __global__ void mut_apply_kernel(BatchView b) {
 // generation counter, stop flag) by the last pass that runs.  One block per
 // instance of the batch.
 
-__global__ void gbest_kernel(BatchView b, int second) {
+__global__ void gbest_kernel(BatchView b, int second, unsigned int* queue, int queues) {
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q < queues; q += blockDim.x) queue[q] = 0;
     const Consts k = b.desc[blockIdx.x].k;
     const SwarmDev d = b.desc[blockIdx.x].d;
     Ctl* c = d.ctl;
@@ -667,10 +670,11 @@ cudaError_t launch_rank_cost(const BatchView& b, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_gbest(const BatchView& b, int second, cudaStream_t st) {
+cudaError_t launch_gbest(const BatchView& b, int second, unsigned int* queue, int queues,
+                         cudaStream_t st) {
     if (b.ninst <= 0) return cudaSuccess;
     const int threads = min(1024, max(128, round_up(b.max_S, 32)));
-    gbest_kernel<<<b.ninst, threads, 0, st>>>(b, second);
+    gbest_kernel<<<b.ninst, threads, 0, st>>>(b, second, queue, queues);
     return cudaGetLastError();
 }
 
