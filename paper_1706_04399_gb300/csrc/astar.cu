@@ -26,7 +26,6 @@
 //  * C[i][j] = C[j][i] = g * unit_mm; blocked_cost where a viewpoint lies
 //    outside the grid or in an occupied voxel, or the cap was exhausted.
 #include <climits>
-#include <vector>
 
 #include "common.cuh"
 
@@ -533,6 +532,26 @@ __global__ void cc_flatten_kernel(long long nv, int* parent) {
         if (parent[v] >= 0) parent[v] = cc_find(parent, static_cast<int>(v));
 }
 
+// The viewpoint pairs (i, j), i < j, row by row (block i).
+__global__ void pairs_kernel(int n, int2* __restrict__ pairs) {
+    const int i = blockIdx.x;
+    const long long first = static_cast<long long>(i) * (2LL * n - i - 1) / 2;
+    for (int j = i + 1 + threadIdx.x; j < n; j += blockDim.x)
+        pairs[first + j - i - 1] = make_int2(i, j);
+}
+
+// Counts the pairs flagged for a second search into *count, and lists them
+// (in whatever order) when `list` is given.
+__global__ void retry_kernel(const int* __restrict__ retry, const int2* __restrict__ pairs,
+                             long long np, unsigned* count, int2* __restrict__ list) {
+    for (long long k = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; k < np;
+         k += static_cast<long long>(gridDim.x) * blockDim.x)
+        if (retry[k]) {
+            const unsigned at = atomicAdd(count, 1u);
+            if (list) list[at] = pairs[k];
+        }
+}
+
 __global__ void zero_diagonal_kernel(int* C, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) C[static_cast<size_t>(i) * n + i] = 0;
@@ -648,11 +667,9 @@ int dpso_voxel_occupancy(const double* boxes_dev, int32_t m, const dpso_astar_pa
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const AstarGrid gr = grid_of(ap);
     const long long nv = static_cast<long long>(gr.nx) * gr.ny * gr.nz;
-    unsigned char* core = nullptr;
-    if (cudaMallocAsync(&core, nv, s) != cudaSuccess) {
-        cudaGetLastError();
-        return DPSO_ERR_NO_MEMORY;
-    }
+    Scratch scratch;
+    if (scratch.acquire(nv, s) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
+    unsigned char* const core = static_cast<unsigned char*>(scratch.p);
     int R = 0;
     while ((R + 1) * (R + 1) <= ap->inflate_r2) ++R;
     const int blocks = static_cast<int>(std::min<long long>((nv + 255) / 256, 65536));
@@ -662,8 +679,8 @@ int dpso_voxel_occupancy(const double* boxes_dev, int32_t m, const dpso_astar_pa
         voxel_inflate_kernel<<<blocks, 256, 0, s>>>(gr, ap->inflate_r2, R, core, occ_dev);
         e = cudaGetLastError();
     }
-    cudaFreeAsync(core, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) scratch.release();  // (the stream was waited for)
     return e == cudaSuccess ? DPSO_OK : DPSO_ERR_CUDA;
 }
 
@@ -675,37 +692,35 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     if (n > DPSO_MAX_N) return DPSO_ERR_RANGE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const long long np = static_cast<long long>(n) * (n - 1) / 2;
-    std::vector<int2> pairs;
-    pairs.reserve(static_cast<size_t>(np));
-    for (int i = 0; i < n; ++i)
-        for (int j = i + 1; j < n; ++j) pairs.push_back(make_int2(i, j));
-    int *vox = nullptr, *retry = nullptr, *err = nullptr, *comp = nullptr;
-    unsigned* queue = nullptr;
-    int2* dpairs = nullptr;
     const long long nv = static_cast<long long>(ap->dims[0]) * ap->dims[1] * ap->dims[2];
-    auto cleanup = [&](int code) {
-        cudaFreeAsync(comp, s);
-        cudaFreeAsync(vox, s);
-        cudaFreeAsync(retry, s);
-        cudaFreeAsync(err, s);
-        cudaFreeAsync(dpairs, s);
-        cudaFreeAsync(queue, s);
-        cudaStreamSynchronize(s);
-        return code;
+    // one allocation: error word, queue and retry count; viewpoint voxels;
+    // components; pairs; retry flags
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+        const size_t here = at;
+        at += (bytes + 255) / 256 * 256;
+        return here;
     };
-    if (cudaMallocAsync(&vox, sizeof(int) * n, s) != cudaSuccess ||
-        cudaMallocAsync(&retry, sizeof(int) * std::max<long long>(np, 1), s) != cudaSuccess ||
-        cudaMallocAsync(&err, sizeof(int), s) != cudaSuccess ||
-        cudaMallocAsync(&comp, sizeof(int) * nv, s) != cudaSuccess ||
-        cudaMallocAsync(&dpairs, sizeof(int2) * std::max<long long>(np, 1), s) != cudaSuccess) {
-        cudaGetLastError();
-        return cleanup(DPSO_ERR_NO_MEMORY);
-    }
+    const size_t oHead = place(3 * sizeof(int)), oVox = place(sizeof(int) * n),
+                 oComp = place(sizeof(int) * nv), oPairs = place(sizeof(int2) * np),
+                 oRetry = place(sizeof(int) * np);
+    Scratch scratch, more;  // (each waits for the stream before it is released)
+    if (scratch.acquire(at, s) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
+    unsigned char* const base = static_cast<unsigned char*>(scratch.p);
+    int* const err = reinterpret_cast<int*>(base + oHead);
+    unsigned* const queue = reinterpret_cast<unsigned*>(err + 1);
+    unsigned* const again = reinterpret_cast<unsigned*>(err + 2);
+    int* const vox = reinterpret_cast<int*>(base + oVox);
+    int* const comp = reinterpret_cast<int*>(base + oComp);
+    int2* const dpairs = reinterpret_cast<int2*>(base + oPairs);
+    int* const retry = reinterpret_cast<int*>(base + oRetry);
     const AstarGrid gr = grid_of(ap);
-    cudaError_t e = cudaMemsetAsync(retry, 0, sizeof(int) * std::max<long long>(np, 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
-    if (e == cudaSuccess && np > 0)
-        e = cudaMemcpyAsync(dpairs, pairs.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, s);
+    cudaError_t e = np > 0 ? cudaMemsetAsync(retry, 0, sizeof(int) * np, s) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 3 * sizeof(int), s);
+    if (e == cudaSuccess && np > 0) {
+        pairs_kernel<<<n - 1, 128, 0, s>>>(n, dpairs);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) {
         viewpoint_voxel_kernel<<<(n + 127) / 128, 128, 0, s>>>(gr, xyz_dev, n, occ_dev, vox);
         e = cudaGetLastError();
@@ -758,10 +773,8 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
         W.err = err;
         A.final_pass = false;
         if (e == cudaSuccess && np > 0) {
-            e = cudaMallocAsync(&queue, sizeof(unsigned), s);
-            if (e == cudaSuccess) e = cudaMemsetAsync(queue, 0, sizeof(unsigned), s);
             W.queue = queue;
-            if (e == cudaSuccess) e = run_warp_pass(W, s);
+            e = run_warp_pass(W, s);
         }
     } else {
         // pass 1: every pair, room for a short search
@@ -773,32 +786,36 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
         if (e == cudaSuccess && np > 0) e = run_pass(A, dpairs, static_cast<int>(np), kBudget, s);
     }
     // pass 2: the pairs that need more room, searched again from the start
-    std::vector<int> flags(static_cast<size_t>(np));
     if (e == cudaSuccess && np > 0 && !A.final_pass) {
-        e = cudaMemcpyAsync(flags.data(), retry, sizeof(int) * np, cudaMemcpyDeviceToHost, s);
+        const int blocks = static_cast<int>(std::min<long long>((np + 255) / 256, 4096));
+        unsigned count = 0;
+        retry_kernel<<<blocks, 256, 0, s>>>(retry, dpairs, np, again, nullptr);
+        e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&count, again, sizeof(count), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        std::vector<int2> again;
-        for (long long k = 0; k < np; ++k)
-            if (flags[k]) again.push_back(pairs[k]);
-        if (e == cudaSuccess && !again.empty()) {
-            e = cudaMemcpyAsync(dpairs, again.data(), sizeof(int2) * again.size(),
-                                cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess && count > 0) {
+            e = more.acquire(sizeof(int2) * count, s);
+            int2* const list = static_cast<int2*>(more.p);
+            if (e == cudaSuccess) e = cudaMemsetAsync(again, 0, sizeof(unsigned), s);
+            if (e == cudaSuccess) {
+                retry_kernel<<<blocks, 256, 0, s>>>(retry, dpairs, np, again, list);
+                e = cudaGetLastError();
+            }
             A.max_exp = ap->max_expansions;
             A.final_pass = true;
             A.heap_cap = 26 * ap->max_expansions + 1;
             A.map_bits = map_bits_for(A.heap_cap);
             A.retry = nullptr;
-            if (e == cudaSuccess)
-                e = run_pass(A, dpairs, static_cast<int>(again.size()), kBudget, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // `again` is read by the copy
+            if (e == cudaSuccess) e = run_pass(A, list, static_cast<int>(count), kBudget, s);
         }
     }
     int herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaErrorMemoryAllocation) return cleanup(DPSO_ERR_NO_MEMORY);
-    if (e != cudaSuccess) return cleanup(DPSO_ERR_CUDA);
-    return cleanup(herr & 2 ? DPSO_ERR_RANGE : DPSO_OK);
+    if (e == cudaErrorMemoryAllocation) return DPSO_ERR_NO_MEMORY;
+    if (e != cudaSuccess) return DPSO_ERR_CUDA;
+    return herr & 2 ? DPSO_ERR_RANGE : DPSO_OK;
 }
 
 }  // extern "C"
