@@ -10,8 +10,9 @@
 // FP32), and the slab test divides six times per pair and box.  A filter in
 // FP32 with an error bound decides nearly every (pair, box); the FP64 test runs
 // on what it leaves open, so the matrix is that of the FP64 test alone.  At
-// n = 1992 with 20 boxes the kernel takes 0.18 ms, 3.32 without the filter;
-// what is left is the FP64 distance and its square root, and the filter.
+// n = 1992 with 20 boxes the kernel took 3.32 ms without the filter, 0.18 with
+// it and FP64 lengths, and 0.13 with lengths in pairs of FP32 numbers (below),
+// FP64 only next to a rounding tie; what is left is the filter.
 #include <math.h>
 
 #include "common.cuh"
@@ -93,6 +94,59 @@ __device__ __forceinline__ int filter_box(const Axis (&ax)[3], const float (&lo)
     return !open && gap > w ? 1 : 2;
 }
 
+// A coordinate as the sum of two FP32 numbers (off by at most 2^-48 of it).
+struct Split {
+    float hi, lo;
+};
+
+__device__ __forceinline__ Split split(double v) {
+    const float hi = static_cast<float>(v);
+    return Split{hi, static_cast<float>(__dsub_rn(v, static_cast<double>(hi)))};
+}
+
+// 1000 |q - p| rounded to the nearest integer, in pairs of FP32 numbers (sums
+// with their rounding error, products with theirs by FMA), where the result is
+// not near a tie; -1: not decided.  With M the largest coordinate magnitude,
+// the differences are off by some 2^-46 M and everything after by some 2^-44
+// of itself, so the length r in mm by less than (r + 1000 M) 2^-40; a tie
+// closer than 2^8 times that (and 2^-20) is left to FP64, whose own error is
+// far below.  Lengths past 2^22 mm, and anything not finite, are left too.
+__device__ __forceinline__ int length_mm(const Split (&p)[3], const Split (&q)[3], float mag) {
+    float sh = 0.f, sl = 0.f;  // the sum of squares
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float a = __fsub_rn(q[k].hi, p[k].hi);  // d = a + e, normalised to h + l
+        const float bb = __fsub_rn(a, q[k].hi);
+        const float e = __fadd_rn(
+            __fsub_rn(__fsub_rn(q[k].hi, __fsub_rn(a, bb)), __fadd_rn(p[k].hi, bb)),
+            __fsub_rn(q[k].lo, p[k].lo));
+        const float h = __fadd_rn(a, e), l = __fsub_rn(e, __fsub_rn(h, a));
+        const float m = __fmul_rn(h, h);
+        const float ml = __fmaf_rn(2.f * h, l, __fmaf_rn(h, h, -m));
+        const float t = __fadd_rn(sh, m);  // sh + m and its error
+        const float tb = __fsub_rn(t, sh);
+        const float te = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, tb)), __fsub_rn(m, tb));
+        sl = __fadd_rn(sl, __fadd_rn(te, ml));
+        sh = t;
+    }
+    if (!(sh < 1.76e7f)) return -1;  // 4.19 km squared, as (2^22 mm)^2
+    if (sh < 1e-20f) return sh == 0.f && sl == 0.f ? 0 : -1;
+    const float y = rsqrtf(sh);
+    const float r0 = __fmul_rn(sh, y);
+    const float res = __fadd_rn(__fmaf_rn(-r0, r0, sh), sl);  // (s - r0^2), r0 within 2^-21
+    const float r1 = __fmul_rn(res, __fmul_rn(0.5f, y));
+    // one more step for the remainder's own square
+    const float r2 = __fmaf_rn(-__fmul_rn(r1, r1), __fmul_rn(0.5f, y), r1);
+    const float vh = __fmul_rn(r0, 1000.f);
+    const float vl = __fadd_rn(__fmaf_rn(r0, 1000.f, -vh), __fmul_rn(r2, 1000.f));
+    const float n = rintf(vh);
+    const float f = __fadd_rn(__fsub_rn(vh, n), vl);  // the distance from n, small
+    const float g = rintf(f);
+    const float away = fabsf(__fsub_rn(fabsf(__fsub_rn(f, g)), 0.5f));
+    if (!(away > 0x1p-20f + (vh + 1000.f * mag) * 0x1p-32f)) return -1;
+    return static_cast<int>(n) + static_cast<int>(g);
+}
+
 // One thread per (i, j) with i < j inside 32 x 32 tiles of the upper triangle,
 // four pairs per thread; boxes are staged in shared memory in chunks.  The
 // tile is mirrored through shared memory, so both halves are written in rows.
@@ -106,6 +160,7 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
     __shared__ double sbox[kBoxes * 6];
     __shared__ float slo[kBoxes][3], shi[kBoxes][3], smag[kBoxes];
     __shared__ int tile[kTile][kTile + 1];
+    __shared__ Split rows[kTile][3];  // the tile's row points
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
     const int tid = ty * kTile + tx;
     const int j = bj + tx;
@@ -117,6 +172,11 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
         qf[k] = static_cast<float>(q[k]);
     }
     bool bad = false;
+    if (tid < 3 * kTile && bi + tid / 3 < n) {
+        const double v = xyz[3 * (size_t)bi + tid];
+        bad = !isfinite(v);  // (every point is a row of its diagonal tile)
+        rows[tid / 3][tid % 3] = split(v);
+    }
     unsigned blocked = 0;  // bit s: pair s
     for (int b0 = 0; b0 < m; b0 += kBoxes) {
         const int cnt = min(kBoxes, m - b0);
@@ -171,40 +231,44 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
             blocked |= static_cast<unsigned>(hit) << s;
         }
     }
-    int vals[4];
+    __syncthreads();
+    Split qs[3];
+    float qmag = 0.f;
 #pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        qs[k] = split(q[k]);
+        qmag = fmaxf(qmag, fabsf(qf[k]));
+    }
+#pragma unroll 2
     for (int s = 0; s < 4; ++s) {
-        const int i = bi + ty + 8 * s;
-        vals[s] = 0;
-        if (i >= n) continue;
-        double p[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            p[k] = xyz[3 * (size_t)i + k];
-            bad = bad || !isfinite(p[k]);  // (every point is a row of its diagonal tile)
+        const int r0 = ty + 8 * s, i = bi + r0;
+        int v = 0;
+        if (i < n && j < n && i < j) {
+            const Split ps[3] = {rows[r0][0], rows[r0][1], rows[r0][2]};
+            const float mag =
+                fmaxf(fmaxf(qmag, fabsf(ps[0].hi)), fmaxf(fabsf(ps[1].hi), fabsf(ps[2].hi)));
+            long long c = length_mm(ps, qs, mag);
+            if (c < 0) {
+                const double* p = xyz + 3 * (size_t)i;
+                const double dx = __dsub_rn(q[0], p[0]);
+                const double dy = __dsub_rn(q[1], p[1]);
+                const double dz = __dsub_rn(q[2], p[2]);
+                double acc = __dmul_rn(dx, dx);
+                acc = __dadd_rn(acc, __dmul_rn(dy, dy));
+                acc = __dadd_rn(acc, __dmul_rn(dz, dz));
+                c = __double2ll_rn(__dmul_rn(1000.0, __dsqrt_rn(acc)));
+            }
+            if (blocked >> s & 1) c += penalty;
+            if (c > DPSO_COST_MAX) {
+                atomicOr(err, 2);
+                c = DPSO_COST_MAX;
+            }
+            v = static_cast<int>(c);
         }
-        if (j >= n || i >= j) continue;
-        const double dx = __dsub_rn(q[0], p[0]);
-        const double dy = __dsub_rn(q[1], p[1]);
-        const double dz = __dsub_rn(q[2], p[2]);
-        double acc = __dmul_rn(dx, dx);
-        acc = __dadd_rn(acc, __dmul_rn(dy, dy));
-        acc = __dadd_rn(acc, __dmul_rn(dz, dz));
-        long long c = __double2ll_rn(__dmul_rn(1000.0, __dsqrt_rn(acc))) +
-                      ((blocked >> s & 1) ? (long long)penalty : 0LL);
-        if (c > DPSO_COST_MAX) {
-            atomicOr(err, 2);
-            c = DPSO_COST_MAX;
-        }
-        vals[s] = static_cast<int>(c);
+        if (i < n && j < n && i <= j) C[(size_t)i * ldc + j] = v;  // (0 on the diagonal)
+        tile[r0][tx] = v;
     }
     if (bad) atomicOr(err, 1);
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int i = bi + ty + 8 * s;
-        if (i < n && j < n && i <= j) C[(size_t)i * ldc + j] = vals[s];  // (0 on the diagonal)
-        tile[ty + 8 * s][tx] = vals[s];
-    }
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < 4; ++s) {  // row bj + r of the lower half, columns bi ..

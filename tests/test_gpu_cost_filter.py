@@ -66,3 +66,14 @@ def test_magnitudes(scale, offset):
     rng = np.random.default_rng(11)
     _check(rng.uniform(0, 20, size=(120, 3)) * scale + offset,
            _boxes(rng, 30, 20.0, 2.0) * scale + offset)
+
+
+@pytest.mark.parametrize("unit", [0.0005, 0.001, 0.0015, 0.25, 1.0 / 1024])
+def test_lengths_at_rounding_ties(unit):
+    # lattices whose lengths in mm fall on or next to half-integers
+    rng = np.random.default_rng(21)
+    xyz = rng.integers(0, 4000, size=(180, 3)) * unit
+    xyz[:60, 1:] = 0.0
+    _check(xyz, np.zeros((0, 6)))
+    xyz[60:90] += rng.integers(-3, 4, size=(30, 3)) * 2.0 ** -40
+    _check(xyz, np.zeros((0, 6)))
