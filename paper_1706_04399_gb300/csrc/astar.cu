@@ -271,12 +271,12 @@ __global__ void astar_pairs_kernel(AstarArgs A) {
 // The same search with one warp per pair and the whole state in shared
 // memory, for searches that stay small (which, with the squared-distance
 // heuristic, is nearly all of them).  Per warp:
-//   map:  kWarpSlots slots (voxel | closed bit, best g), linear probing with
+//   map:  kSlots slots (voxel | closed bit, best g), linear probing with
 //         lanes inserting concurrently by 64-bit CAS (nothing is deleted
 //         within a search, so a lane that finds an empty slot knows its voxel
 //         is not further along);
-//   open: an append-only array of keys (f << 42 | h << 24 | voxel), popped
-//         entries overwritten with ~0.  Keys of live entries are distinct
+//   open: an array of keys (f << 42 | h << 24 | voxel) in no order, a popped
+//         entry replaced by the last one.  Keys of live entries are distinct
 //         (a voxel is pushed again only with a smaller g), so the pop is a
 //         warp-wide minimum and its owner lane is unique.
 // A pop, the closed test, the goal and cap tests are uniform over the warp;
@@ -287,12 +287,26 @@ __global__ void astar_pairs_kernel(AstarArgs A) {
 // that would outgrow the map or the open array is left to the global pass
 // (retry flag).  Host-checked bounds keep f < 2^22, h < 2^18 and every grid
 // dimension at most 256.
-constexpr int kWarpSlots = 2048;         // map slots per warp
-constexpr int kWarpOpen = 2048;          // open entries per warp
-constexpr int kWarpDistinct = 1900;      // inserts before a search hands over
-constexpr int kWarpsPerBlock = 7;        // 7 x 32 KB of shared memory per block
 constexpr unsigned long long kEmptySlot = ~0ull;
 constexpr unsigned kClosed = 1u << 30;   // closed bit of a slot's voxel word
+
+// Sizes of a warp's map and open list, and the warps that then fit on an SM's
+// shared memory in one block.
+// The first pass's slots: 14 searches per SM instead of 7 hide more of each
+// expansion's dependent steps (facade, 400 viewpoints: 2.46 -> 1.94 ms for the
+// whole call; 512 slots send too many searches on, 2.59); the few that outgrow
+// it run again with 2048.
+constexpr int kSmall = 1024;
+template <int SLOTS>
+struct WarpSearch {
+    static constexpr int kSlots = SLOTS;                  // map slots
+    static constexpr int kOpen = SLOTS;                   // open entries
+    static constexpr int kDistinct = SLOTS - SLOTS / 14;  // inserts before a search hands over
+    static constexpr int kBytes = (kSlots + kOpen) * 8;
+    static constexpr int kWarps = 224 * 1024 / kBytes;
+    static constexpr int kBits = SLOTS == 2048 ? 11 : (SLOTS == 1024 ? 10 : 9);
+    static_assert(1 << kBits == SLOTS, "a power of two");
+};
 
 struct WarpArgs {
     AstarGrid gr;
@@ -301,6 +315,7 @@ struct WarpArgs {
     const int* comp;
     const int2* pairs;
     int npairs;
+    const unsigned* count;  // when set, *count pairs instead of npairs
     unsigned* queue;  // next pair (zero on entry)
     int a1, a2, a3;
     long long unit_mm;
@@ -327,31 +342,34 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long v)
     return (static_cast<unsigned long long>(mhi) << 32) | mlo;
 }
 
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) astar_warp_kernel(WarpArgs A) {
+template <int SLOTS>
+__global__ void __launch_bounds__(32 * WarpSearch<SLOTS>::kWarps) astar_warp_kernel(WarpArgs A) {
+    using W = WarpSearch<SLOTS>;
     extern __shared__ unsigned long long sm_astar[];
     const int lane = threadIdx.x & 31;
-    unsigned long long* const open = sm_astar + (threadIdx.x >> 5) * (kWarpOpen + kWarpSlots);
-    unsigned long long* const map = open + kWarpOpen;
+    unsigned long long* const open = sm_astar + (threadIdx.x >> 5) * (W::kOpen + W::kSlots);
+    unsigned long long* const map = open + W::kOpen;
     const int nx = A.gr.nx, ny = A.gr.ny, nz = A.gr.nz;
     const int nxy = nx * ny;
     // this lane's neighbour offset (lanes 0..25; the 27 offsets minus the centre)
     const int d = lane < 13 ? lane : lane + 1;
     const int ddx = d % 3 - 1, ddy = (d / 3) % 3 - 1, ddz = d / 9 - 1;
     const int step = A.a1 * ddx * ddx + A.a2 * ddy * ddy + A.a3 * ddz * ddz;
-    auto slot0 = [](int c) { return (static_cast<unsigned>(c) * 2654435761u) >> 21; };  // 11 bits
+    auto slot0 = [](int c) { return (static_cast<unsigned>(c) * 2654435761u) >> (32 - W::kBits); };
     auto cw = [](unsigned long long e) { return static_cast<int>((e >> 32) & (kClosed - 1)); };
     constexpr unsigned long long kClosedBit = static_cast<unsigned long long>(kClosed) << 32;
+    const int npairs = A.count ? static_cast<int>(*A.count) : A.npairs;
     for (;;) {
         int k = 0;
         if (lane == 0) k = static_cast<int>(atomicAdd(A.queue, 1u));
         k = __shfl_sync(0xffffffffu, k, 0);
-        if (k >= A.npairs) break;
+        if (k >= npairs) break;
         const int2 pr = A.pairs[k];
         const int s = A.vox[pr.x], t = A.vox[pr.y];
         long long result = -1;
         bool handover = false;
         if (s >= 0 && t >= 0 && A.comp[s] == A.comp[t]) {
-            for (int i = lane; i < kWarpSlots; i += 32) map[i] = kEmptySlot;
+            for (int i = lane; i < W::kSlots; i += 32) map[i] = kEmptySlot;
             const int tx = t % nx, ty = (t / nx) % ny, tz = t / nxy;
             const int sx = s % nx, sy = (s / nx) % ny, sz = s / nxy;
             const int tc = pack_xyz(tx, ty, tz), sc = pack_xyz(sx, sy, sz);
@@ -380,7 +398,9 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) astar_warp_kernel(WarpArg
                 }
                 const unsigned long long top = warp_min_key(mine);
                 if (top == ~0ull) break;  // the open list is exhausted
-                if (mine == top) open[at] = ~0ull;
+                // the last entry takes its place (the list is in no order)
+                --len;
+                if (mine == top) open[at] = open[len];
                 const int c = static_cast<int>(top & 0xffffffu);
                 const int h = static_cast<int>((top >> 24) & 0x3ffffu);
                 const int g = static_cast<int>(top >> 42) - h;
@@ -388,8 +408,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) astar_warp_kernel(WarpArg
                 // bounded all the same, and a miss hands the pair over
                 unsigned sv = slot0(c);
                 unsigned long long e = map[sv];
-                for (int probe = 1; probe < kWarpSlots && cw(e) != c; ++probe) {
-                    sv = (sv + 1) & (kWarpSlots - 1);
+                for (int probe = 1; probe < W::kSlots && cw(e) != c; ++probe) {
+                    sv = (sv + 1) & (W::kSlots - 1);
                     e = map[sv];
                 }
                 __syncwarp();
@@ -405,7 +425,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) astar_warp_kernel(WarpArg
                 }
                 if (expanded >= A.max_exp) break;  // cap: blocked
                 ++expanded;
-                if (distinct + 26 > kWarpDistinct || len + 26 > kWarpOpen) {
+                if (distinct + 26 > W::kDistinct || len + 26 > W::kOpen) {
                     handover = true;
                     break;
                 }
@@ -419,10 +439,10 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) astar_warp_kernel(WarpArg
                     const unsigned long long want =
                         (static_cast<unsigned long long>(u) << 32) | static_cast<unsigned>(gu);
                     unsigned su = slot0(u);
-                    // fewer than kWarpSlots voxels are ever inserted, so an
-                    // empty slot ends the probe within kWarpSlots steps
+                    // fewer than W::kSlots voxels are ever inserted, so an
+                    // empty slot ends the probe within W::kSlots steps
                     lost = true;
-                    for (int probe = 0; probe < kWarpSlots; ++probe) {
+                    for (int probe = 0; probe < W::kSlots; ++probe) {
                         unsigned long long cur = map[su];
                         if (cur == kEmptySlot) {
                             cur = atomicCAS(map + su, kEmptySlot, want);
@@ -440,7 +460,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) astar_warp_kernel(WarpArg
                             lost = false;
                             break;
                         }
-                        su = (su + 1) & (kWarpSlots - 1);
+                        su = (su + 1) & (W::kSlots - 1);
                     }
                     if (push) {
                         const int hu =
@@ -592,16 +612,17 @@ bool warp_pass_fits(const dpso_astar_params* ap) {
            gmax + hmax < (1ll << 22);
 }
 
-cudaError_t run_warp_pass(const WarpArgs& W, cudaStream_t st) {
+template <int SLOTS>
+cudaError_t run_warp_pass(const WarpArgs& A, cudaStream_t st) {
+    using W = WarpSearch<SLOTS>;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int smem = kWarpsPerBlock * (kWarpOpen + kWarpSlots) * static_cast<int>(sizeof(unsigned long long));
-    if (e == cudaSuccess)
-        e = raise_smem_limit(astar_warp_kernel, smem);
+    constexpr int smem = W::kWarps * W::kBytes;
+    if (e == cudaSuccess) e = raise_smem_limit(astar_warp_kernel<SLOTS>, smem);
     if (e != cudaSuccess) return e;
-    const int blocks = std::max(1, std::min(sms, (W.npairs + kWarpsPerBlock - 1) / kWarpsPerBlock));
-    astar_warp_kernel<<<blocks, 32 * kWarpsPerBlock, smem, st>>>(W);
+    const int blocks = std::max(1, std::min(sms, (A.npairs + W::kWarps - 1) / W::kWarps));
+    astar_warp_kernel<SLOTS><<<blocks, 32 * W::kWarps, smem, st>>>(A);
     return cudaGetLastError();
 }
 
@@ -693,30 +714,30 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const long long np = static_cast<long long>(n) * (n - 1) / 2;
     const long long nv = static_cast<long long>(ap->dims[0]) * ap->dims[1] * ap->dims[2];
-    // one allocation: error word, queue and retry count; viewpoint voxels;
-    // components; pairs; retry flags
+    // one allocation: error word, two queues and the count of pairs to search
+    // again; viewpoint voxels; components; pairs; flags and list of those
     size_t at = 0;
     auto place = [&](size_t bytes) {
         const size_t here = at;
         at += (bytes + 255) / 256 * 256;
         return here;
     };
-    const size_t oHead = place(3 * sizeof(int)), oVox = place(sizeof(int) * n),
+    const size_t oHead = place(4 * sizeof(int)), oVox = place(sizeof(int) * n),
                  oComp = place(sizeof(int) * nv), oPairs = place(sizeof(int2) * np),
-                 oRetry = place(sizeof(int) * np);
+                 oRetry = place(sizeof(int) * np), oMore = place(sizeof(int2) * np);
     Scratch scratch, more;  // (each waits for the stream before it is released)
     if (scratch.acquire(at, s) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
     unsigned char* const base = static_cast<unsigned char*>(scratch.p);
     int* const err = reinterpret_cast<int*>(base + oHead);
     unsigned* const queue = reinterpret_cast<unsigned*>(err + 1);
-    unsigned* const again = reinterpret_cast<unsigned*>(err + 2);
+    unsigned* const again = reinterpret_cast<unsigned*>(err + 3);
     int* const vox = reinterpret_cast<int*>(base + oVox);
     int* const comp = reinterpret_cast<int*>(base + oComp);
-    int2* const dpairs = reinterpret_cast<int2*>(base + oPairs);
+    int2* dpairs = reinterpret_cast<int2*>(base + oPairs);
     int* const retry = reinterpret_cast<int*>(base + oRetry);
     const AstarGrid gr = grid_of(ap);
     cudaError_t e = np > 0 ? cudaMemsetAsync(retry, 0, sizeof(int) * np, s) : cudaSuccess;
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 3 * sizeof(int), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 4 * sizeof(int), s);
     if (e == cudaSuccess && np > 0) {
         pairs_kernel<<<n - 1, 128, 0, s>>>(n, dpairs);
         e = cudaGetLastError();
@@ -751,9 +772,11 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     A.err = err;
     constexpr size_t kBudget = size_t(4) << 30;  // scratch bytes per pass
     A.retry = retry;
+    const int retry_blocks = static_cast<int>(std::max<long long>(1, std::min<long long>((np + 255) / 256, 4096)));
     if (warp_pass_fits(ap)) {
         // pass 1: every pair, one warp per search in shared memory, the full
-        // cap; searches that outgrow the warp's map or open array are retried
+        // cap; searches that outgrow the warp's map or open array are searched
+        // again with larger ones, then in pass 2
         WarpArgs W{};
         W.gr = gr;
         W.occ = occ_dev;
@@ -774,7 +797,20 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
         A.final_pass = false;
         if (e == cudaSuccess && np > 0) {
             W.queue = queue;
-            e = run_warp_pass(W, s);
+            e = run_warp_pass<kSmall>(W, s);
+            // the searches that outgrew the small map, with the large one
+            int2* const list = reinterpret_cast<int2*>(base + oMore);
+            if (e == cudaSuccess) {
+                retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, dpairs, np, again, list);
+                e = cudaGetLastError();
+            }
+            if (e == cudaSuccess) e = cudaMemsetAsync(retry, 0, sizeof(int) * np, s);
+            W.pairs = list;
+            W.count = again;
+            W.queue = queue + 1;
+            if (e == cudaSuccess) e = run_warp_pass<2048>(W, s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(again, 0, sizeof(unsigned), s);
+            dpairs = list;
         }
     } else {
         // pass 1: every pair, room for a short search
@@ -787,9 +823,8 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     }
     // pass 2: the pairs that need more room, searched again from the start
     if (e == cudaSuccess && np > 0 && !A.final_pass) {
-        const int blocks = static_cast<int>(std::min<long long>((np + 255) / 256, 4096));
         unsigned count = 0;
-        retry_kernel<<<blocks, 256, 0, s>>>(retry, dpairs, np, again, nullptr);
+        retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, dpairs, np, again, nullptr);
         e = cudaGetLastError();
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&count, again, sizeof(count), cudaMemcpyDeviceToHost, s);
@@ -799,7 +834,7 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
             int2* const list = static_cast<int2*>(more.p);
             if (e == cudaSuccess) e = cudaMemsetAsync(again, 0, sizeof(unsigned), s);
             if (e == cudaSuccess) {
-                retry_kernel<<<blocks, 256, 0, s>>>(retry, dpairs, np, again, list);
+                retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, dpairs, np, again, list);
                 e = cudaGetLastError();
             }
             A.max_exp = ap->max_expansions;
