@@ -159,9 +159,12 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
     // are read in a few steps, are faster without (n = 400, 1024 tours: a swarm's
     // generations 8 % slower with them).
     constexpr bool kLists = ST == kCtaRows || ST == kGlobal;
-    constexpr int kBatch = 4;                       // partners a thread has in flight
-    // threads per group of the choice of T' (see the head of the file)
-    constexpr int kGroup = NT / 16;
+    // partners a thread has in flight (n = 400, 1024 tours, whole call: 1 3.39
+    // ms, 2 3.32, 4 3.73, 8 about 6: the rare path is unrolled with the common one)
+    constexpr int kBatch = 2;
+    // threads per group of the choice of T' (see the head of the file): eight
+    // groups (16 groups 3.65 ms, 32 more)
+    constexpr int kGroup = NT >= 256 ? 32 : (NT >= 128 ? 16 : 8);
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned long long s_key[2][kW];  // the warps' best, by pass parity
     __shared__ int s_lo[kW], s_hi[kW];
@@ -852,7 +855,8 @@ cudaError_t launch_cfg(const TwoOptBatch& b, int cap, int num_sms, cudaStream_t 
 // Launch configurations: for tours of up to max_n viewpoints (and, with
 // `few`, launches of at most that many tours per SM): threads per tour,
 // staging, list entries.  Measured on GB300 (random grid, facade and bridge
-// tours to 2-optimality, whole call, ms; warp = each warp stages its rows):
+// tours to 2-optimality, whole call, ms; warp = each warp stages its rows;
+// with four partners in flight and 16 groups):
 //   n     tours  matrix 256  warp 64 / 128  CTA 128 / 256 / 512   C 128 / 256
 //   157   256    0.70        1.02 / 0.80                          0.80 / -
 //   157   1024   1.31        1.25 / 1.43                          1.39 / -
@@ -872,8 +876,8 @@ constexpr int kAny = INT_MAX;
 constexpr ListConfig kConfigs[] = {
     {160, 2, 256, kMatrix, 512},        {220, 1, 256, kMatrix, 512},
     {512, 2, 256, kGlobal, 512},        {512, 4, 128, kWarpRows, 512},
-    {512, kAny, 64, kWarpRows, 512},    {1200, 1, 256, kGlobal, 1024},
-    {1200, kAny, 128, kCtaRows, 1024},  {5000, kAny, 256, kCtaRows, 1024},
+    {512, kAny, 64, kWarpRows, 1024},    {1200, 1, 256, kGlobal, 1024},
+    {1200, kAny, 128, kCtaRows, 1024},  {5000, kAny, 256, kCtaRows, 2048},
     {DPSO_MAX_N, kAny, 512, kGlobal, 1024},
 };
 constexpr int kNumConfigs = sizeof(kConfigs) / sizeof(kConfigs[0]);
