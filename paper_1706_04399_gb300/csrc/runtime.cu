@@ -440,10 +440,10 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
     };
     // followed by the 2-opt's neighbour lists
     const size_t head = (sizeof(Head) + 255) / 256 * 256;
-    const bool lists = kind == 0 && near_used(n, count, sms);
+    bool lists = kind == 0 && near_used(n, count, sms);
     Scratch room;
-    if (room.acquire(head + (lists ? near_bytes(n) : 0), st) != cudaSuccess)
-        return DPSO_ERR_NO_MEMORY;
+    if (lists) lists = room.acquire(head + near_bytes(n), st) == cudaSuccess;
+    if (!room.p && room.acquire(head, st) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
     Head* const scratch = static_cast<Head*>(room.p);
     int* err = &scratch->err;
     int herr = 0;

@@ -64,8 +64,9 @@ struct Active {
     int fail = 0;       // status the request failed with while running
 };
 
-// Device bytes one request holds while active (the arrays dpso_init
-// allocates, each rounded to the 512-byte allocation granule) plus the
+// Device bytes one request may hold while active (the arrays dpso_init
+// allocates, and for a 2-opt the row-shifted cost copies that a shape pinned on
+// a batch would add, more than its neighbour lists) plus the
 // transient buffers of its admission (viewpoints, boxes, the unpadded cost
 // matrix).  Only the planning estimate for admission, not an allocator.
 size_t request_footprint(int n, int m, int S, int T, int flags) {
@@ -74,8 +75,9 @@ size_t request_footprint(int n, int m, int S, int T, int flags) {
     size_t hist = 1024;
     while (hist < static_cast<size_t>(T)) hist *= 2;
     size_t b = a(n * ldc * 4);                                       // C
-    if ((flags & DPSO_FLAG_TWO_OPT) && dpso::two_opt_tiled_rows(n) > 0)
-        b += a(static_cast<size_t>(4) * n * dpso::shifted_ld(n) * 4);  // shifted copies
+    if (flags & DPSO_FLAG_TWO_OPT)  // shifted copies; past the tiled kernel's limit the lists
+        b += dpso::two_opt_tiled_rows(n) > 0 ? a(static_cast<size_t>(4) * n * dpso::shifted_ld(n) * 4)
+                                             : a(dpso::near_bytes(n));
     b += 3 * a(s * ldn * 2) + a(ldn * 2);                             // X, V, P, G
     b += 3 * a(s * 8) + 2 * a(s) + a(s * 4);                          // F, PF, hash, dup, kept, order
     b += a(hist * 8) + 2 * a(sizeof(SwarmDesc) + 1024);               // history, control, meta
