@@ -15,16 +15,18 @@ value   particle-iterations/s = particles x generations / device time of the
         matrix and swarm resident in HBM; the L2 is flushed between timed
         generations.  For N > 1 each rank runs an independent replica (the
         solver has no exchange step to shard).
-2-opt moves/s  candidate 2-opt pairs the exchange kernel evaluated per second
-        of its own device time (`two_opt_pairs_evaluated_per_s`); the pairs a
-        plain best-improvement scan of the same passes would take are
-        reported beside it.
+2-opt moves/s  candidate 2-opt pairs the exchange kernel decided (evaluated, or
+        excluded by a bound on their row) per second of its own device time
+        (`two_opt_pairs_evaluated_per_s`); the pairs a plain best-improvement
+        scan of the same passes would take are reported beside it.
 e2e     the same metric through dpso_plan from pinned host buffers: copies in,
         cost matrix, initialisation, `steps` generations, best tour out.
-roofline  the 2-opt kernel: 8 bytes of C per candidate pair evaluated (two
-        int32 entries) over its CUDA-event time inside the timed generations,
-        against the L2 read bandwidth measured in this run (the cost matrix is
-        L2-resident; rows are staged from L2).
+roofline  the 2-opt kernel: 8 bytes of C per candidate pair decided (two int32
+        entries, which an excluded pair does not read) over its CUDA-event time
+        inside the timed generations, against the L2 read bandwidth measured in
+        this run (the cost matrix is L2-resident).  The node-swap kernel counts
+        the plain scan's pairs, nearly all of which it need not look at, so it
+        has no such figure.
 fitness_roofline  the tour-fitness kernel (Eq. min) over the swarm's tours:
         4 n bytes of C gathered per tour over its CUDA-event time, against the
         random 4-byte gather rate from an L2-resident buffer measured in this
@@ -466,12 +468,14 @@ def gpu_line(args):
                   for mb in (8, 16, 24)}
         l2 = max(probes.values())
         bpp = BYTES_PER_SWAP_PAIR if node_swap else BYTES_PER_PAIR
-        # bytes of the pairs the kernel evaluated (a pass skips the rows the
-        # last move left unchanged), not of the pairs a plain scan would take
+        # bytes of the pairs the kernel decided, not of the pairs a plain scan
+        # would take (the node swap reports only the latter: no figure)
         achieved = bpp * evaluated / (two_ms / 1e3) / 1e9 if two_ms > 0 else 0.0
-        traffic = None if node_swap else dram_traffic("two_opt_tiled_kernel", inst.name)
+        if node_swap:
+            achieved = 0.0
+        traffic = None if node_swap else dram_traffic("two_opt_list_kernel", inst.name)
         roofline = {
-            "kernel": "node_swap_tiled_kernel" if node_swap else "two_opt_tiled_kernel",
+            "kernel": "node_swap_kernel" if node_swap else "two_opt_list_kernel",
             "bound": "l2", "bytes_per_pair": bpp, "pairs_evaluated": evaluated,
             "achieved": achieved, "peak": l2,
             "unit": "GB/s", "frac": achieved / l2 if l2 else None,
@@ -529,7 +533,7 @@ def gpu_line(args):
             "ms_per_step": dev_ms_max / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "i32", "data": "synthetic",
             "config": config,
-            # the metric's "2-opt moves/s": candidate pairs the kernel evaluated
+            # the metric's "2-opt moves/s": candidate pairs the kernel decided
             "two_opt_pairs_evaluated_per_s": evaluated / (two_ms / 1e3) if two_ms > 0 else 0.0,
             "two_opt_pairs_evaluated": evaluated,
             # what a plain best-improvement scan of the same passes would take

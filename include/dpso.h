@@ -103,8 +103,9 @@ typedef struct dpso_stats {
     int64_t two_opt_runs;   /* generations in which the edge exchange ran */
     int32_t device_status;  /* sticky device-side error code (DPSO_OK if none) */
     int32_t reserved;
-    int64_t two_opt_evaluated; /* candidate pairs the kernels evaluated, counted up
-                                  to two_opt_pairs: fewer when a pass knows from
+    int64_t two_opt_evaluated; /* candidate pairs the kernels decided (evaluated, or
+                                  excluded by a bound on their row), counted up to
+                                  two_opt_pairs: fewer when a pass knows from
                                   earlier ones that a pair cannot be the best; a
                                   count of this process's work, not saved in a
                                   state.  The node swap reports two_opt_pairs. */
