@@ -1,7 +1,7 @@
 // Edge exchange of Sec. 3.2.3 (best-improvement 2-opt to 2-optimality), the
 // pipelined tiled variant for tours whose 33-row tiles fit in shared memory.
 //
-// Same mathematics and tie order as two_opt.cu:
+// Same mathematics and tie order as two_opt_list.cu:
 //   delta(i, j) = C[x_i][x_j] + C[x_i+1][x_j+1] - C[x_i][x_i+1] - C[x_j][x_j+1],
 //   the applied move is the smallest (delta, i, j) with delta < 0.
 //
