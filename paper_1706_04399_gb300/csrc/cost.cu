@@ -165,7 +165,11 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
     __shared__ int tile[kTile][kTile + 1];
     __shared__ Split rows[kTile][3];  // the tile's row points
     __shared__ float hull[2][2][3];   // of the row and the column points: lowest, highest
-    __shared__ int kept;              // boxes of the chunk that meet the hull of both
+    // Boxes of the chunk that meet the hull of both, by the chunk's parity: a
+    // warp may clear the next chunk's count while another has yet to read this
+    // chunk's; this one's is cleared again two chunks on, after the barriers of
+    // the one between.
+    __shared__ int kept[2];
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
     const int tid = ty * kTile + tx;
     const int j = bj + tx;
@@ -200,9 +204,9 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
         }
     }
     unsigned blocked = 0;  // bit s: pair s
-    for (int b0 = 0; b0 < m; b0 += kBoxes) {
+    for (int b0 = 0, par = 0; b0 < m; b0 += kBoxes, par ^= 1) {
         int cnt = min(kBoxes, m - b0);
-        if (tid == 0) kept = 0;
+        if (tid == 0) kept[par] = 0;
         __syncthreads();
         for (int e = tid; e < cnt * 6; e += kTile * 8) {
             const double v = boxes[6 * (size_t)b0 + e];
@@ -230,7 +234,7 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
                 out = out || fmaxf(hull[0][1][k], hull[1][1][k]) < lo[k] - E ||
                       fminf(hull[0][0][k], hull[1][0][k]) > hi[k] + E;
             if (!out) {
-                const int at = atomicAdd(&kept, 1);
+                const int at = atomicAdd(&kept[par], 1);
                 for (int k = 0; k < 3; ++k) {
                     slo[at][k] = lo[k];
                     shi[at][k] = hi[k];
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(kTile * 8, 2) cost_matrix_kernel(
             }
         }
         __syncthreads();
-        cnt = kept;
+        cnt = kept[par];
 #pragma unroll 1
         for (int s = 0; s < 4; ++s) {
             const int i = bi + ty + 8 * s;
