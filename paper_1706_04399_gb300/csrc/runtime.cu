@@ -898,32 +898,35 @@ struct dpso_batch {
     bool any_two_opt = false;
     std::vector<TwoOptTask> tasks;       // host: every exchanging member, by descending n
     std::vector<dpso_swarm*> owners;     // the members the tasks belong to
-    std::vector<TwoOptClass> cls;
-    unsigned int* queues = nullptr;      // device: a work queue per class
+    // The launch classes and the generation graph over them, whose nodes hold
+    // the classes' device arrays: they are made and freed together.
+    struct Route {
+        std::vector<TwoOptClass> cls;
+        unsigned int* queues = nullptr;  // device: a work queue per class
+        cudaGraphExec_t graph = nullptr;
+    } route;
     std::vector<cudaStream_t> side;      // capture streams of the classes after the first
     std::vector<cudaEvent_t> ev;         // fork, then one join per side stream
     cudaStream_t cap = nullptr;
-    cudaGraphExec_t graph = nullptr;
     cudaStream_t last = nullptr;
 };
 
 namespace {
 
-void free_classes(dpso_batch* b) {
-    for (auto& c : b->cls) {
+void free_route(dpso_batch::Route& r) {
+    if (r.graph) cudaGraphExecDestroy(r.graph);
+    for (auto& c : r.cls) {
         void* bufs[] = {c.tasks, c.toff};
         for (void* p : bufs)
             if (p) cudaFree(p);
     }
-    b->cls.clear();
-    if (b->queues) cudaFree(b->queues);
-    b->queues = nullptr;
+    if (r.queues) cudaFree(r.queues);
+    r = dpso_batch::Route{};
 }
 
 void free_batch(dpso_batch* b) {
     if (!b) return;
-    if (b->graph) cudaGraphExecDestroy(b->graph);
-    free_classes(b);
+    free_route(b->route);
     void* bufs[] = {b->desc, b->off};
     for (void* p : bufs)
         if (p) cudaFree(p);
@@ -966,9 +969,10 @@ int ensure_batch_shifted(dpso_batch* b) {
 
 // Splits the exchanging members into launch classes: runs of members (by
 // descending n) whose default shape and resident CTAs per SM agree, each
-// launched with that shape; or one class with a pinned shape for all.
-int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
-    free_classes(b);
+// launched with that shape; or one class with a pinned shape for all.  The
+// batch's present route stays as it is; what an error leaves in `r` is the
+// caller's to free.
+int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned, dpso_batch::Route& r) {
     const int nt = static_cast<int>(b->tasks.size());
     std::vector<std::pair<int, int>> runs;  // [first, last) task ranges
     std::vector<ShapeKey> keys;
@@ -986,7 +990,7 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
         }
     }
     if (!runs.empty()) {
-        const int st = dalloc(&b->queues, runs.size(), b->last);
+        const int st = dalloc(&r.queues, runs.size(), b->last);
         if (st) return st;
     }
     for (size_t c = 0; c < runs.size(); ++c) {
@@ -1002,17 +1006,17 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
         }
         int st = DPSO_OK;
         if ((st = dalloc(&cl.tasks, cnt, b->last)) || (st = dalloc(&cl.toff, cnt + 1, b->last))) {
-            b->cls.push_back(cl);
+            r.cls.push_back(cl);
             return st;
         }
-        b->cls.push_back(cl);
+        r.cls.push_back(cl);
         CK(cudaMemcpyAsync(cl.tasks, b->tasks.data() + first, sizeof(TwoOptTask) * cnt,
                            cudaMemcpyHostToDevice, b->last));
         CK(cudaMemcpyAsync(cl.toff, toff.data(), sizeof(int) * (cnt + 1), cudaMemcpyHostToDevice,
                            b->last));
         CK(cudaStreamSynchronize(b->last));  // the host vectors go out of scope
-        TwoOptBatch& tb = b->cls.back().tb;
-        tb = TwoOptBatch{cl.tasks, cl.toff, cnt, toff.back(), max_n, shifted, 0, b->queues + c};
+        TwoOptBatch& tb = r.cls.back().tb;
+        tb = TwoOptBatch{cl.tasks, cl.toff, cnt, toff.back(), max_n, shifted, 0, r.queues + c};
         tb.kind = keys[c].kind;
         if (keys[c].kind == 1) {
             // node swap: the launch follows max_n
@@ -1023,12 +1027,12 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
         }
     }
     // one capture stream and one join event per class after the first
-    while (b->side.size() + 1 < b->cls.size()) {
+    while (b->side.size() + 1 < r.cls.size()) {
         cudaStream_t s = nullptr;
         CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
         b->side.push_back(s);
     }
-    while (b->ev.size() < b->cls.size()) {
+    while (b->ev.size() < r.cls.size()) {
         cudaEvent_t e = nullptr;
         CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         b->ev.push_back(e);
@@ -1039,45 +1043,51 @@ int build_classes(dpso_batch* b, const dpso_two_opt_shape* pinned) {
 // One generation of every member: the particle update, mutation, gbest, the
 // exchange order, then the classes' 2-opt launches side by side (forked from
 // and joined back into `st`), then the second gbest pass.
-cudaError_t enqueue_batch_classes(dpso_batch* b, cudaStream_t st) {
+cudaError_t enqueue_batch_classes(dpso_batch* b, dpso_batch::Route& r, cudaStream_t st) {
     cudaError_t e = launch_move(b->bv, st);
     if (e == cudaSuccess) e = launch_mutation(b->bv, st);
     if (e == cudaSuccess)
-        e = launch_gbest(b->bv, 0, b->queues, static_cast<int>(b->cls.size()), st);
+        e = launch_gbest(b->bv, 0, r.queues, static_cast<int>(r.cls.size()), st);
     if (e != cudaSuccess || !b->any_two_opt) return e;
     if (b->bv.total > b->num_sms) e = launch_rank_cost(b->bv, st);
-    if (e == cudaSuccess && b->cls.size() > 1) e = cudaEventRecord(b->ev[0], st);
-    for (size_t c = 1; c < b->cls.size() && e == cudaSuccess; ++c) {
+    if (e == cudaSuccess && r.cls.size() > 1) e = cudaEventRecord(b->ev[0], st);
+    for (size_t c = 1; c < r.cls.size() && e == cudaSuccess; ++c) {
         cudaStream_t s = b->side[c - 1];
         e = cudaStreamWaitEvent(s, b->ev[0], 0);
-        if (e == cudaSuccess) e = launch_two_opt(b->cls[c].tb, b->num_sms, s);
+        if (e == cudaSuccess) e = launch_two_opt(r.cls[c].tb, b->num_sms, s);
         if (e == cudaSuccess) e = cudaEventRecord(b->ev[c], s);
     }
-    if (e == cudaSuccess && !b->cls.empty()) {
-        e = launch_two_opt(b->cls[0].tb, b->num_sms, st);
+    if (e == cudaSuccess && !r.cls.empty()) {
+        e = launch_two_opt(r.cls[0].tb, b->num_sms, st);
     }
-    for (size_t c = 1; c < b->cls.size() && e == cudaSuccess; ++c)
+    for (size_t c = 1; c < r.cls.size() && e == cudaSuccess; ++c)
         e = cudaStreamWaitEvent(st, b->ev[c], 0);
     if (e == cudaSuccess) e = launch_gbest(b->bv, 1, nullptr, 0, st);
     return e;
 }
 
-int capture_batch(dpso_batch* b) {
-    if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
+int capture_batch(dpso_batch* b, dpso_batch::Route& r) {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeRelaxed));
-    const cudaError_t e = enqueue_batch_classes(b, b->cap);
+    const cudaError_t e = enqueue_batch_classes(b, r, b->cap);
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return DPSO_ERR_CUDA;
     }
-    const cudaError_t e3 = cudaGraphInstantiate(&b->graph, g, 0);
+    const cudaError_t e3 = cudaGraphInstantiate(&r.graph, g, 0);
     cudaGraphDestroy(g);
     return e3 == cudaSuccess ? DPSO_OK : DPSO_ERR_CUDA;
+}
+
+// Builds the graph over r's classes and, when `st` and that are without error,
+// puts r in the place of the batch's route (no launch of which is running);
+// else frees r and leaves the batch as it was.
+int finish_route(dpso_batch* b, dpso_batch::Route& r, int st) {
+    if (st == DPSO_OK) st = capture_batch(b, r);
+    if (st == DPSO_OK) std::swap(b->route, r);
+    free_route(r);
+    return st;
 }
 
 // Times the list kernel and every tiled shape that fits a class on scratch
@@ -1241,10 +1251,11 @@ int dpso_batch_create(dpso_batch** out, dpso_swarm* const* swarms, int32_t count
         cudaStreamSynchronize(b->last) != cudaSuccess)
         return fail(DPSO_ERR_CUDA);
     b->bv = BatchView{b->desc, b->off, count, off[count], max_ldn, arrays, max_S};
-    if ((st = build_classes(b, nullptr))) return fail(st);
     if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
         return fail(DPSO_ERR_CUDA);
-    if ((st = capture_batch(b))) return fail(st);
+    dpso_batch::Route r;
+    st = build_classes(b, nullptr, r);
+    if ((st = finish_route(b, r, st))) return fail(st);
     *out = b;
     return DPSO_OK;
 }
@@ -1266,7 +1277,7 @@ int dpso_batch_step(dpso_batch* b, int32_t iterations, void* stream) {
         CK(cudaStreamSynchronize(b->last));
         b->last = st;
     }
-    for (int it = 0; it < iterations; ++it) CK(cudaGraphLaunch(b->graph, st));
+    for (int it = 0; it < iterations; ++it) CK(cudaGraphLaunch(b->route.graph, st));
     for (dpso_swarm* s : b->members) s->t_host += iterations;
     return DPSO_OK;
 }
@@ -1281,18 +1292,16 @@ int dpso_batch_autotune(dpso_batch* b, dpso_two_opt_shape* chosen, void* stream)
     const int r0 = ensure_batch_shifted(b);
     if (r0 && r0 != DPSO_ERR_NO_MEMORY) return r0;
     // the classes are built again with the copies; a shape pinned before is timed anew
-    const int r1 = build_classes(b, nullptr);
-    if (r1) return r1;
-    for (auto& cl : b->cls) {
-        const int r = autotune_class(b, cl, st);
-        if (r) return r;
-    }
-    const int r = capture_batch(b);
+    dpso_batch::Route route;
+    int r = build_classes(b, nullptr, route);
+    for (size_t c = 0; r == DPSO_OK && c < route.cls.size(); ++c)
+        r = autotune_class(b, route.cls[c], st);
+    r = finish_route(b, route, r);
     if (r) return r;
     if (chosen) {  // the shape of the class holding the longest tours
         *chosen = dpso_two_opt_shape{0, 0, 0};
-        if (!b->cls.empty()) {
-            const TwoOptBatch& tb = b->cls[0].tb;
+        if (!b->route.cls.empty()) {
+            const TwoOptBatch& tb = b->route.cls[0].tb;
             int rows = tb.rows, tpc = tb.tpc, tg = tb.tg;
             if (rows <= 0) {  // the class runs the default shape for its tours
                 int sms = 0;
@@ -1337,9 +1346,8 @@ int dpso_batch_set_two_opt_shape(dpso_batch* b, const dpso_two_opt_shape* shape)
         const int st = ensure_batch_shifted(b);
         if (st) return st;
     }
-    const int st = build_classes(b, defaults ? nullptr : shape);
-    if (st) return st;
-    return capture_batch(b);
+    dpso_batch::Route r;
+    return finish_route(b, r, build_classes(b, defaults ? nullptr : shape, r));
 }
 
 void dpso_batch_destroy(dpso_batch* b) {
