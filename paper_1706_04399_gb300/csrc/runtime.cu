@@ -441,6 +441,8 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
     // followed by the 2-opt's neighbour lists
     const size_t head = (sizeof(Head) + 255) / 256 * 256;
     bool lists = kind == 0 && near_used(n, count, sms);
+    Head host{};  // read by asynchronous copies: it outlives the scratch's wait
+    host.toff[1] = count;
     Scratch room;
     if (lists) lists = room.acquire(head + near_bytes(n), st) == cudaSuccess;
     if (!room.p && room.acquire(head, st) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
@@ -448,8 +450,6 @@ int exchange_tours(int kind, const int32_t* C_dev, int32_t n, uint16_t* tours_de
     int* err = &scratch->err;
     int herr = 0;
     unsigned long long counters[2] = {0, 0};
-    Head host{};
-    host.toff[1] = count;
     cudaError_t e = cudaMemcpyAsync(scratch, &host, sizeof(Head), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = launch_check_cost_limit(C_dev, n, n, kind ? DPSO_NODE_SWAP_COST_MAX : DPSO_COST_MAX, err, st);
     if (e == cudaSuccess) {
@@ -618,6 +618,7 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
     if ((st = ensure_history(s, 1024))) return fail(st);
     s->d = SwarmDev{s->C,    s->X,   s->V,    s->P,   s->G,    s->F,
                     s->PF,   s->hash, s->dup, s->kept, s->ctl, s->order};
+    SwarmMeta meta{};  // read by an asynchronous copy: it outlives the scratch's wait below
     // error word, back-and-forth orders and tags: scratch of this call
     const size_t orders_at = 256, tags_at = orders_at + 2 * 8 * ldn;
     Scratch scratch;
@@ -650,16 +651,13 @@ int dpso_init(dpso_swarm** out, const int32_t* C_dev, int32_t n, const int32_t* 
     if (herr & 2) return fail(DPSO_ERR_RANGE);
     if (lists && build_near(s->C, k.ldc, n, s->near, ust) != cudaSuccess)
         return fail(DPSO_ERR_CUDA);
-    {
-        SwarmMeta m{};
-        m.desc.k = k;
-        m.desc.d = s->d;
-        m.task = swarm_task(s);
-        m.off[1] = k.S;
-        m.toff[1] = k.S;
-        if (cudaMemcpyAsync(s->meta, &m, sizeof(m), cudaMemcpyHostToDevice, ust) != cudaSuccess)
-            return fail(DPSO_ERR_CUDA);
-    }
+    meta.desc.k = k;
+    meta.desc.d = s->d;
+    meta.task = swarm_task(s);
+    meta.off[1] = k.S;
+    meta.toff[1] = k.S;
+    if (cudaMemcpyAsync(s->meta, &meta, sizeof(meta), cudaMemcpyHostToDevice, ust) != cudaSuccess)
+        return fail(DPSO_ERR_CUDA);
 
     if (launch_init_particles(k, s->d, orders, s->n_det, ust) != cudaSuccess ||
         launch_fitness(s->C, k.ldc, n, s->X, k.ldn, k.S, s->F, ust) != cudaSuccess ||
