@@ -953,16 +953,38 @@ ShapeKey default_shape(int n, int kind) {
 }
 
 // Gives every 2-opt member the row-shifted copies the tiled kernel reads.
-int ensure_batch_shifted(dpso_batch* b) {
+// `made` receives the tasks whose members had none before.
+int ensure_batch_shifted(dpso_batch* b, std::vector<size_t>* made) {
     for (size_t i = 0; i < b->tasks.size(); ++i) {
         if (b->tasks[i].kind != 0) continue;
         dpso_swarm* s = b->owners[i];
+        const bool had = s->Cs != nullptr;
         const int st = ensure_shifted(s);
         if (st) return st;
+        if (!had) made->push_back(i);
         CK(cudaStreamSynchronize(s->last));  // the batch's launches may be on another stream
         b->tasks[i].Cs = s->Cs;
     }
     return DPSO_OK;
+}
+
+// Takes the copies of those of `made` that the batch's route does not read from
+// their members again (no other batch has seen copies that this call made).
+void drop_unread_shifted(dpso_batch* b, const std::vector<size_t>& made) {
+    auto read = [&](size_t task) {  // the classes are runs of the tasks, in order
+        size_t first = 0;
+        for (const auto& c : b->route.cls) {
+            first += c.tb.nprob;
+            if (task < first) return c.tb.kind == 0 && c.tb.rows > 0;
+        }
+        return false;
+    };
+    for (size_t i : made) {
+        if (read(i)) continue;
+        cudaFree(b->owners[i]->Cs);
+        b->owners[i]->Cs = nullptr;
+        b->tasks[i].Cs = nullptr;
+    }
 }
 
 // Splits the exchanging members into launch classes: runs of members (by
@@ -1287,24 +1309,25 @@ int dpso_batch_autotune(dpso_batch* b, dpso_two_opt_shape* chosen, void* stream)
     CK(cudaStreamSynchronize(b->last));
     b->last = st;
     // (without room for the copies only the list kernel can run: nothing to choose)
-    const int r0 = ensure_batch_shifted(b);
-    if (r0 && r0 != DPSO_ERR_NO_MEMORY) return r0;
-    // the classes are built again with the copies; a shape pinned before is timed anew
+    std::vector<size_t> made;
     dpso_batch::Route route;
-    int r = build_classes(b, nullptr, route);
-    for (size_t c = 0; r == DPSO_OK && c < route.cls.size(); ++c)
-        r = autotune_class(b, route.cls[c], st);
-    r = finish_route(b, route, r);
+    int r = ensure_batch_shifted(b, &made);
+    if (r == DPSO_OK || r == DPSO_ERR_NO_MEMORY) {
+        // the classes are built again with the copies; a shape pinned before is timed anew
+        r = build_classes(b, nullptr, route);
+        for (size_t c = 0; r == DPSO_OK && c < route.cls.size(); ++c)
+            r = autotune_class(b, route.cls[c], st);
+        r = finish_route(b, route, r);
+    }
+    drop_unread_shifted(b, made);
     if (r) return r;
     if (chosen) {  // the shape of the class holding the longest tours
         *chosen = dpso_two_opt_shape{0, 0, 0};
         if (!b->route.cls.empty()) {
             const TwoOptBatch& tb = b->route.cls[0].tb;
             int rows = tb.rows, tpc = tb.tpc, tg = tb.tg;
-            if (rows <= 0) {  // the class runs the default shape for its tours
-                int sms = 0;
-                CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
-                two_opt_default_shape(tb.max_n, tb.total, sms, &rows, &tpc, &tg);
+            if (rows <= 0) {  // the class runs the list kernel
+                two_opt_default_shape(tb.max_n, tb.total, b->num_sms, &rows, &tpc, &tg);
             } else {
                 if (tpc <= 0) tpc = two_opt_tiled_tpc(tb.max_n, rows);
                 if (tg <= 0) tg = two_opt_tiled_tg(tb.max_n, rows, tpc);
@@ -1340,12 +1363,12 @@ int dpso_batch_set_two_opt_shape(dpso_batch* b, const dpso_two_opt_shape* shape)
             return DPSO_ERR_ARG;
     }
     CK(cudaStreamSynchronize(b->last));
-    if (!defaults) {
-        const int st = ensure_batch_shifted(b);
-        if (st) return st;
-    }
+    std::vector<size_t> made;
     dpso_batch::Route r;
-    return finish_route(b, r, build_classes(b, defaults ? nullptr : shape, r));
+    int st = defaults ? DPSO_OK : ensure_batch_shifted(b, &made);
+    if (st == DPSO_OK) st = finish_route(b, r, build_classes(b, defaults ? nullptr : shape, r));
+    if (st) drop_unread_shifted(b, made);
+    return st;
 }
 
 void dpso_batch_destroy(dpso_batch* b) {

@@ -1,4 +1,5 @@
-"""A batch call that fails leaves the batch as it was."""
+"""A batch call that fails leaves the batch as it was, and one that succeeds
+keeps no memory that the batch does not read."""
 import numpy as np
 import pytest
 
@@ -47,3 +48,25 @@ def test_failed_autotune_keeps_the_route():
         assert np.array_equal(got[key], want[key]), key
     batch.close()
     sw.close()
+
+
+def test_autotune_keeps_no_copies_for_the_list_kernel():
+    inst = inputs.random_instance(900, 2, 32)  # row-shifted copies of 13 MB
+    C = cost_matrix_gpu(inst)
+    p = dpso.default_params(swarm=64)
+    free = []
+    for _ in range(2):  # (the first batch loads the kernels)
+        sw = dpso.Swarm(C, inst.n, inst.tags, p, 8)
+        batch = dpso.Batch([sw])
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+        rows, tpc, tg = batch.autotune()
+        assert rows in (32, 30, 24, 16, 8) and tpc in (1, 2, 4) and tg in (1, 2)
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+        batch.set_two_opt_shape(rows, tpc, tg)  # (the copies are made again)
+        batch.step(1)
+        batch.close()
+        sw.close()
+    # random tours, 32 moves each: the list kernel is several times faster
+    assert free[3] > free[2] - (8 << 20)
