@@ -681,7 +681,9 @@ def batched_line(args):
         "batched": {"one_per_launch_value": solo_value, "speedup": value / solo_value,
                     "one_per_launch_ms_per_step": ms_solo / args.steps,
                     "identical_states": identical,
-                    "two_opt_shapes": (f"autotuned; last class ({rows}, {tpc}, {tg})" if args.autotune
+                    "two_opt_shapes": (f"autotuned; the longest class's fastest tiled shape is ({rows}, "
+                                        f"{tpc}, {tg}), in use where the list kernel is slower"
+                                        if args.autotune
                                        else "each class's default shape"),
                     "two_opt_pairs_per_s_over_step": pairs / (ms_batch / 1e3),
                     # every member advances one generation per replay of the

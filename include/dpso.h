@@ -350,19 +350,24 @@ typedef struct {
     int32_t tiles_in_flight;
 } dpso_two_opt_shape;
 
-/* Picks the 2-opt kernel and launch shape for this batch by timing the list
- * kernel and every tiled shape that fits on scratch copies of the members'
- * current tours (at most 32 moves per tour each; best called right after
- * creation).  Results do not depend on the choice.  *chosen (may be NULL)
- * receives the tiled shape in use, or where the list kernel was faster the
- * tiled kernel's default shape (dpso_two_opt_default_shape).  Synchronises
- * `stream`. */
+/* Picks the 2-opt kernel and launch shape for each class of this batch by
+ * timing the list kernel and every tiled shape that fits on scratch copies of
+ * the members' current tours (at most 32 moves per tour each; best called
+ * right after creation).  Results do not depend on the choice.  *chosen (may
+ * be NULL) receives the fastest tiled shape for the longest 2-opt members.  It
+ * is the one in use only where it was faster than the list kernel, so it is
+ * no shape to pin again: pinning it puts every member on the tiled kernel.
+ * Where there was no room for the copies that the tiled kernel reads, nothing
+ * is timed and *chosen is the default shape (dpso_two_opt_default_shape).
+ * The copies are kept only for members whose class runs a tiled shape.  On an
+ * error the batch goes on as before the call.  Synchronises `stream`. */
 int dpso_batch_autotune(dpso_batch *b, dpso_two_opt_shape *chosen, void *stream);
 /* Sets the 2-opt launch shape by hand (NULL or all zero: the list kernel).
  * DPSO_ERR_ARG when the shape is not one of the above or does not fit in
  * shared memory for the longest member; DPSO_ERR_NO_MEMORY without room for
  * the row-shifted cost copies the tiled kernel reads (made at the first
- * pinned shape).  Results do not depend on the shape.
+ * pinned shape).  On an error the batch goes on as before the call.  Results
+ * do not depend on the shape.
  * Synchronises the batch's stream. */
 int dpso_batch_set_two_opt_shape(dpso_batch *b, const dpso_two_opt_shape *shape);
 /* The tiled 2-opt kernel's default launch shape for a launch over `count` tours

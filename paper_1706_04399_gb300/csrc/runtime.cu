@@ -887,6 +887,7 @@ struct dpso_batch {
         TwoOptTask* tasks = nullptr;  // device, the class's members by descending n
         int* toff = nullptr;          // device, tour offsets (nprob + 1)
         TwoOptBatch tb{};
+        dpso_two_opt_shape tiled{0, 0, 0};  // the fastest tiled shape an autotune timed
     };
     int device = 0, num_sms = 0;
     std::vector<dpso_swarm*> members;
@@ -1111,8 +1112,8 @@ int finish_route(dpso_batch* b, dpso_batch::Route& r, int st) {
 }
 
 // Times the list kernel and every tiled shape that fits a class on scratch
-// copies of its tours (gates ignored, at most kProbeMoves moves per tour) and
-// keeps the fastest.
+// copies of its tours (gates ignored, at most kProbeMoves moves per tour),
+// keeps the fastest and notes the fastest tiled one.
 int autotune_class(dpso_batch* b, dpso_batch::TwoOptClass& cl, cudaStream_t st) {
     constexpr int kProbeMoves = 32;
     if (cl.tb.kind != 0 || cl.tb.nprob <= 0 || !cl.tb.shifted ||
@@ -1162,8 +1163,7 @@ int autotune_class(dpso_batch* b, dpso_batch::TwoOptClass& cl, cudaStream_t st) 
         cudaStreamSynchronize(st) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
         cudaEventCreate(&e1) != cudaSuccess)
         return cleanup(DPSO_ERR_CUDA);
-    float best = 1e30f;
-    int rows_b = 0, tpc_b = 0, tg_b = 0;
+    float list_ms = 1e30f, tiled_ms = 1e30f;
     constexpr int kShapes[4][2] = {{1, 1}, {2, 1}, {4, 1}, {1, 2}};  // (tours per CTA, tiles)
     for (int rows : {0, 32, 30, 24, 16, 8}) {  // 0: the list kernel
         for (const auto& sh : kShapes) {
@@ -1198,18 +1198,18 @@ int autotune_class(dpso_batch* b, dpso_batch::TwoOptClass& cl, cudaStream_t st) 
                 cudaEventSynchronize(e1) != cudaSuccess ||
                 cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
                 return cleanup(DPSO_ERR_CUDA);
-            if (ms < best) {
-                best = ms;
-                rows_b = rows;
-                tpc_b = tpc;
-                tg_b = tg;
+            if (rows == 0) {
+                list_ms = ms;
+            } else if (ms < tiled_ms) {
+                tiled_ms = ms;
+                cl.tiled = dpso_two_opt_shape{rows, tpc, tg};
             }
         }
     }
-    if (rows_b > 0) {
-        cl.tb.rows = rows_b;
-        cl.tb.tpc = tpc_b;
-        cl.tb.tg = tg_b;
+    if (tiled_ms < list_ms) {
+        cl.tb.rows = cl.tiled.rows;
+        cl.tb.tpc = cl.tiled.tours_per_cta;
+        cl.tb.tg = cl.tiled.tiles_in_flight;
     }
     return cleanup(DPSO_OK);
 }
@@ -1321,18 +1321,15 @@ int dpso_batch_autotune(dpso_batch* b, dpso_two_opt_shape* chosen, void* stream)
     }
     drop_unread_shifted(b, made);
     if (r) return r;
-    if (chosen) {  // the shape of the class holding the longest tours
+    if (chosen) {  // of the class holding the longest 2-opt tours
         *chosen = dpso_two_opt_shape{0, 0, 0};
-        if (!b->route.cls.empty()) {
-            const TwoOptBatch& tb = b->route.cls[0].tb;
-            int rows = tb.rows, tpc = tb.tpc, tg = tb.tg;
-            if (rows <= 0) {  // the class runs the list kernel
-                two_opt_default_shape(tb.max_n, tb.total, b->num_sms, &rows, &tpc, &tg);
-            } else {
-                if (tpc <= 0) tpc = two_opt_tiled_tpc(tb.max_n, rows);
-                if (tg <= 0) tg = two_opt_tiled_tg(tb.max_n, rows, tpc);
-            }
-            *chosen = dpso_two_opt_shape{rows, tpc, tg};
+        for (const auto& c : b->route.cls) {
+            if (c.tb.kind != 0) continue;
+            *chosen = c.tiled;
+            if (chosen->rows == 0)  // (none was timed)
+                two_opt_default_shape(c.tb.max_n, c.tb.total, b->num_sms, &chosen->rows,
+                                      &chosen->tours_per_cta, &chosen->tiles_in_flight);
+            break;
         }
     }
     return DPSO_OK;

@@ -461,7 +461,9 @@ class Batch:
         _check(lib().dpso_batch_step(self._h, iterations, _stream(stream)), "dpso_batch_step")
 
     def autotune(self, stream=None) -> tuple[int, int, int]:
-        """Chosen 2-opt launch shape: (tile height, tours per CTA, tiles in flight)."""
+        """Times the 2-opt kernels and keeps the fastest; returns the fastest tiled shape
+        (tile height, tours per CTA, tiles in flight) of the longest members, which is
+        in use only where it was faster than the list kernel."""
         sh = dpso_two_opt_shape()
         _check(lib().dpso_batch_autotune(self._h, ctypes.byref(sh), _stream(stream)),
                "dpso_batch_autotune")
