@@ -19,9 +19,19 @@
 //    is then a lower bound on the pairs it owns;
 //  * takes the smallest best; stale positions below the best that is not stale
 //    scan the pairs they own first.
-// Before its first scan a position is stale at -2 s (costs are not negative).
 // Owning by the larger s keeps stale positions few: the ones that many others
 // would pair with own those pairs themselves.
+//
+// The first pass looks at every pair.  With M_i(j) = C[x_i][x_j] the four costs
+// above are M_i-1(j), M_i+1(j), M_i(j-1) and M_i(j+1): a thread that holds
+// neighbouring positions j and walks all i gathers one cost per pair, from the
+// row of x_i+1 that the block staged meanwhile, and has the others from the
+// steps before and from its neighbour lane.  Against
+// a scan of every position's row, one swap per tour, whole call: 999 viewpoints,
+// 30 tours 1143 -> 395 us; 1500 viewpoints, 700 tours 8.9 -> 1.8 ms; 2000
+// viewpoints, 304 tours 8.3 -> 1.5 ms.  What bounds it: issue, six instructions
+// a pair and the gather; with one tour per SM, the chain of n steps of some 500
+// cycles each.
 //
 // The costs of a scanned position's pairs lie in three rows of C, those of the
 // six positions in ten; they are staged in shared memory (short tours: the
@@ -42,24 +52,47 @@ using namespace tiled;
 constexpr unsigned long long kExact = 0x8000;
 constexpr unsigned long long kNone = ~0ull;
 constexpr int kNodeSwapMaxN = 4497;  // longer tours are refused
+constexpr int kThreadsPerSm = 640;  // the register budget's resident threads
 constexpr int kRowsStaged = 10;  // two swapped positions, two on each side
 
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(smem)), "l"(gmem)
                  : "memory");
 }
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(smem)), "l"(gmem)
+                 : "memory");
+}
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// At most `Pending` of this thread's latest copy groups are still in flight.
+template <int Pending>
+__device__ __forceinline__ void cp_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(Pending) : "memory");
+}
 
 __host__ __device__ constexpr int mat_ld(int n) { return n | 1; }
 
 // Where costs are read: the whole matrix in shared memory, staged rows (three
-// per warp, ten at least), or C itself (the longest tours).
+// per warp, ten at least), or C itself (the longest tours; the first pass's rows
+// lie in the room of bestof, which it fills at its end, and in up to four rows
+// more, as many as leave two blocks their room on an SM).
 enum Costs { kMatrix, kStaged, kGlobal };
 
+__host__ __device__ constexpr int rows_beside(int n, int warps, Costs costs) {
+    if (costs == kStaged) return 3 * warps > kRowsStaged ? 3 * warps : kRowsStaged;
+    const int room = (112 * 1024 - 20 * n) / (4 * n);
+    return room > 4 ? 4 : (room < 2 ? 2 : room);
+}
+// Rows the first pass stages: pairs of them, at most four.
+__host__ __device__ constexpr int ring_rows(int n, int warps, Costs costs) {
+    const int rows = rows_beside(n, warps, costs) + (costs == kGlobal ? 2 : 0);
+    return rows > 8 ? 8 : rows / 2 * 2;
+}
+
 __host__ __device__ constexpr size_t staged_words(int n, int warps, Costs costs) {
-    const size_t rows = 3 * warps > kRowsStaged ? 3 * warps : kRowsStaged;
     return (costs == kMatrix ? static_cast<size_t>(n) * mat_ld(n)
-                             : (costs == kStaged ? rows * n : 0)) + 3;
+                             : static_cast<size_t>(rows_beside(n, warps, costs)) * n) + 3;
 }
 
 constexpr size_t swap_smem(int n, int warps, Costs costs) {
@@ -68,10 +101,14 @@ constexpr size_t swap_smem(int n, int warps, Costs costs) {
                (sizeof(unsigned long long) + 2 * sizeof(int) + 2 * sizeof(uint16_t));
 }
 
-template <int NT, Costs COSTS>
-__global__ void __launch_bounds__(NT) node_swap_kernel(TwoOptBatch b) {
+// NT threads solve one tour; COLS: positions a thread holds in the first pass.
+template <int NT, Costs COSTS, int COLS>
+__global__ void __launch_bounds__(NT, COLS > 8 ? 3 : (NT == 96 ? 5 : kThreadsPerSm / NT))
+    node_swap_kernel(TwoOptBatch b) {
     constexpr int kW = NT / 32;
     constexpr bool kFull = COSTS == kMatrix, kRows = COSTS == kStaged;
+    constexpr int kCols = COLS;
+    constexpr int kNobody = 0xffff;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned long long s_exact[2][kW], s_stale[2][kW], s_six[2][kW][6];
     __shared__ int s_item, s_rows;
@@ -117,9 +154,7 @@ __global__ void __launch_bounds__(NT) node_swap_kernel(TwoOptBatch b) {
         if (tid == 0) s_rows = 0;
         __syncthreads();
         for (int i = tid; i < n; i += NT) {
-            const int s = dd[prev(i)] + dd[i];
-            ss[i] = s;
-            bestof[i] = s > 0 ? pack_key(-2 * s, 0, 0) : kNone;
+            ss[i] = dd[prev(i)] + dd[i];
         }
         long long f = a.cost[p];
         int moves = 0, passes = 0, par = 0;
@@ -157,7 +192,162 @@ __global__ void __launch_bounds__(NT) node_swap_kernel(TwoOptBatch b) {
             return (static_cast<unsigned long long>(mh) << 32) | ml;
         };
 
-        unsigned long long exact = kNone, stale = 0;  // the smallest of each kind
+        unsigned long long exact, stale;  // the smallest of each kind
+        auto smallest = [&]() {  // over all positions; one barrier
+            exact = kNone;
+            stale = kNone;
+            for (int i = tid; i < n; i += NT) {
+                const unsigned long long v = bestof[i];
+                if (v & kExact) exact = min(exact, v);
+                else stale = min(stale, v);
+            }
+            exact = warp_min(exact);
+            stale = warp_min(stale);
+            if (lane == 0) {
+                s_exact[par][warp] = exact;
+                s_stale[par][warp] = stale;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < kW; ++w) {
+                exact = min(exact, s_exact[par][w]);
+                stale = min(stale, s_stale[par][w]);
+            }
+            par ^= 1;
+        };
+
+        // The first pass, NT * kCols positions j at a time.  Of the pairs with
+        // an s_i no larger than s_j (those that j owns, and ties) the best one's i
+        // goes to rows[j], except where i and j are neighbours: kApart in the place
+        // of C's diagonal keeps those from improving.  Two rows are taken per
+        // barrier, the next ones meanwhile on their way.
+        constexpr int kApart = 1 << 29;  // twice it: no less than any s_i + s_j
+        // The q-th row that a walk over i = 0 .. n-1 needs, q = i + 2 for x_i+1.
+        auto walk_city = [&](int q) { return static_cast<int>(X[q == 0 ? n - 1 : (q > n ? 0 : q - 1)]); };
+        const int steps = (n + 3) / 2, ahead = kFull ? 0 : ring_rows(b.max_n, kW, COSTS) / 2;
+        const bool wide = ((reinterpret_cast<size_t>(C) | (4 * static_cast<size_t>(ldc))) & 15) == 0 &&
+                          (n & 3) == 0;  // rows (and the staged ones) start on 16 bytes
+        auto stage = [&](int t, int slot) {
+            if constexpr (!kFull) {
+                if (t < steps) {
+                    const int* r0 = C + static_cast<size_t>(walk_city(2 * t)) * ldc;
+                    const int* r1 = C + static_cast<size_t>(walk_city(2 * t + 1)) * ldc;
+                    int* const to = mat + 2 * slot * n;
+                    if (wide) {
+                        for (int c = 4 * tid; c < n; c += 4 * NT) {
+                            cp_async16(&to[c], r0 + c);
+                            cp_async16(&to[n + c], r1 + c);
+                        }
+                    } else {
+#pragma unroll 4
+                        for (int c = tid; c < n; c += NT) {
+                            cp_async4(&to[c], r0 + c);
+                            cp_async4(&to[n + c], r1 + c);
+                        }
+                    }
+                }
+                cp_commit();
+            }
+        };
+        for (int c0 = 0; c0 < n; c0 += NT * kCols) {
+            const int j0 = c0 + tid * kCols;
+            // (best: s_j + the best delta so far; past n: nothing is owned)
+            int xj[kCols], sj[kCols], up[kCols], mid[kCols], best[kCols], bi[kCols];
+#pragma unroll
+            for (int k = 0; k < kCols; ++k) {
+                const int j = j0 + k;
+                xj[k] = X[j < n ? j : 0];  // (position n - 1 is followed by 0)
+                sj[k] = j < n ? ss[j] : -1;
+                best[k] = sj[k];
+                bi[k] = kNobody;
+                up[k] = mid[k] = 0;
+            }
+            // the neighbours of the warp's first and last position
+            const int xe = X[lane == 0 ? (j0 == 0 ? n - 1 : min(j0, n) - 1)
+                                       : (j0 + kCols < n ? j0 + kCols : 0)];
+            int mid_e = 0;
+            auto look = [&](int i, const int (&u)[kCols], const int (&m)[kCols], int m_e,
+                            const int (&w)[kCols]) {
+                const int si = ss[i];
+                int left = __shfl_up_sync(0xffffffffu, m[kCols - 1], 1);
+                int right = __shfl_down_sync(0xffffffffu, m[0], 1);
+                if (lane == 0) left = m_e;
+                if (lane == 31) right = m_e;
+#pragma unroll
+                for (int k = 0; k < kCols; ++k) {
+                    const int d = u[k] + w[k] + (k > 0 ? m[k - 1] : left) +
+                                  (k + 1 < kCols ? m[k + 1] : right) - si;
+                    // (of equal deltas the smaller i has the smaller key)
+                    const bool better = sj[k] >= si && d < best[k];
+                    best[k] = better ? d : best[k];
+                    bi[k] = better ? i : bi[k];
+                }
+            };
+            for (int t = 0; t + 1 < ahead; ++t) stage(t, t);
+            for (int t = 0, slot = 0; t < steps; ++t) {
+                const int u0 = walk_city(2 * t), u1 = walk_city(2 * t + 1);
+                const int* const r0 = kFull ? mat + u0 * ld : mat + 2 * slot * n;
+                const int* const r1 = kFull ? mat + u1 * ld : r0 + n;
+                if constexpr (!kFull) {
+                    if (ahead > 3) cp_wait<2>();
+                    else if (ahead > 2) cp_wait<1>();
+                    else cp_wait<0>();
+                    // (by the thread that copied the word)
+                    if ((wide ? u0 / 4 : u0) % NT == tid) mat[2 * slot * n + u0] = kApart;
+                    if ((wide ? u1 / 4 : u1) % NT == tid) mat[2 * slot * n + n + u1] = kApart;
+                    __syncthreads();  // rows 2t, 2t + 1 are there, those before no longer read
+                    stage(t + ahead - 1, slot == 0 ? ahead - 1 : slot - 1);
+                }
+                auto read = [&](const int* row, int u, int x) {
+                    const int v = row[x];
+                    return kFull && x == u ? kApart : v;
+                };
+                int a0[kCols], a1[kCols], e0 = 0, e1 = 0;
+#pragma unroll
+                for (int k = 0; k < kCols; ++k) {
+                    a0[k] = read(r0, u0, xj[k]);
+                    a1[k] = read(r1, u1, xj[k]);
+                }
+                if (lane == 0 || lane == 31) {
+                    e0 = read(r0, u0, xe);
+                    e1 = read(r1, u1, xe);
+                }
+                if (t > 0) {
+                    look(2 * t - 2, up, mid, mid_e, a0);
+                    if (2 * t - 1 < n) look(2 * t - 1, mid, a0, e0, a1);
+                }
+#pragma unroll
+                for (int k = 0; k < kCols; ++k) {
+                    up[k] = a0[k];
+                    mid[k] = a1[k];
+                }
+                mid_e = e1;
+                if (++slot == ahead) slot = 0;
+            }
+#pragma unroll
+            for (int k = 0; k < kCols; ++k)
+                if (j0 + k < n) rows[j0 + k] = static_cast<uint16_t>(bi[k]);
+            if (!kFull) cp_wait_all();
+            __syncthreads();  // the staged rows are no longer read
+        }
+        // ... and with the pairs of neighbours that j owns, its best.
+        for (int j = tid; j < n; j += NT) {
+            auto at = [&](int p0, int q0) {
+                const int u = X[p0], w = X[q0];
+                return kFull ? mat[u * ld + w] : C[static_cast<size_t>(u) * ldc + w];
+            };
+            const int from[3] = {rows[j], prev(j), next(j)};
+            unsigned long long v = kNone;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int i = from[q];
+                if (i == kNobody || (q > 0 && !owns(ss[j], j, ss[i], i))) continue;
+                v = min(v, key_of(at(prev(i), j) + at(next(i), j) + at(i, prev(j)) + at(i, next(j)) -
+                                      ss[i] - ss[j] + adjacent(i, j), i, j));
+            }
+            bestof[j] = v;
+        }
+        smallest();  // (a thread reads what it wrote; the barrier is for the others)
         for (;;) {
             if (max_moves > 0 && moves >= max_moves) break;
             if (moves >= guard) {
@@ -202,26 +392,7 @@ __global__ void __launch_bounds__(NT) node_swap_kernel(TwoOptBatch b) {
                 }
                 __syncthreads();
                 if (tid == 0) s_rows = 0;
-                exact = kNone;
-                stale = kNone;
-                for (int i = tid; i < n; i += NT) {
-                    const unsigned long long v = bestof[i];
-                    if (v & kExact) exact = min(exact, v);
-                    else stale = min(stale, v);
-                }
-                exact = warp_min(exact);
-                stale = warp_min(stale);
-                if (lane == 0) {
-                    s_exact[par][warp] = exact;
-                    s_stale[par][warp] = stale;
-                }
-                __syncthreads();
-#pragma unroll
-                for (int w = 0; w < kW; ++w) {
-                    exact = min(exact, s_exact[par][w]);
-                    stale = min(stale, s_stale[par][w]);
-                }
-                par ^= 1;
+                smallest();
             }
             ++passes;
             if (exact == kNone) break;
@@ -380,9 +551,9 @@ __global__ void __launch_bounds__(NT) node_swap_kernel(TwoOptBatch b) {
     }
 }
 
-template <int NT, Costs COSTS>
+template <int NT, Costs COSTS, int COLS>
 cudaError_t launch_nt(const TwoOptBatch& b, int num_sms, cudaStream_t st) {
-    auto* kern = node_swap_kernel<NT, COSTS>;
+    auto* kern = node_swap_kernel<NT, COSTS, COLS>;
     const size_t smem = swap_smem(b.max_n, NT / 32, COSTS);
     cudaError_t e = raise_smem_limit(kern, smem);
     if (e != cudaSuccess) return e;
@@ -413,18 +584,34 @@ namespace {
 //   400   256    -                     5367 / 4496 / 4448         -
 //   400   512    -                     5883 / 4993 / 5495         -
 //   400   1024   -                     7648 / 9351 / 9645         -
-//   999   300    -                     33572 / 28211 / 25103      26252
-//   2000  300    -                     281220 / 208503 / 175774   153964
-// (the tiled kernel that scanned every pair took 46 ms for 512 tours at 400)
+// and with the first pass by column blocks (one swap only in brackets; a block
+// is NT * cols positions; 128 threads with 8, past 1024 viewpoints 12 of them):
+//   620   600    -                     - / 8586 (345) / 8785 (402)      -
+//   800   600    -                     - / 13586 (732) / 13703 (521)    -
+//   999   150    -                     - / - / 14257 (390)        12451 (426)
+//   999   300    -                     - / - / 16364 (486)        16612 (648)
+//   999   600    -                     - / 36213 (1379) / 32533 (869)   32756 (1225)
+//   1200  150    -                     - / - / 19800 (726, cols 8) 17786 (502)
+//   1200  300    -                     - / - / 21406 (616)        24647 (768)
+//   1200  600    -                     - / 50215 (1764) / 41118 (1150)  47664 (1452)
+//   1500  150    -                     - / - / 29363 (905, cols 8) 27310 (623)
+//   1500  300    -                     - / - / 32566 (799)        40545 (982)
+//   1500  760    -                     - / - / 92768 (1841)       111130 (2235)
+//   2000  300    -                     - / - / 175774 (cols 8)    153964
+// From 800 to 1024 viewpoints, one tour per SM at most, C is the faster for whole
+// descents and the staged rows for few swaps; the line lies where both agree.
+// (The tiled kernel that scanned every pair took 46 ms for 512 tours at 400.)
 struct SwapConfig {
     int max_n, few, threads;
     Costs costs;
+    int cols;
 };
 constexpr int kAny = INT_MAX;
 constexpr SwapConfig kConfigs[] = {
-    {64, kAny, 64, kMatrix},  {100, kAny, 128, kMatrix},  {160, 2, 128, kMatrix},
-    {220, 1, 128, kMatrix},   {1500, 2, 128, kStaged},    {1500, 5, 96, kStaged},
-    {600, kAny, 64, kStaged}, {1500, kAny, 128, kStaged}, {kNodeSwapMaxN, kAny, 256, kGlobal},
+    {64, kAny, 64, kMatrix, 2},     {100, kAny, 128, kMatrix, 2},   {160, 2, 128, kMatrix, 2},
+    {220, 1, 128, kMatrix, 2},      {1024, 2, 128, kStaged, 8},     {1500, 1, 256, kGlobal, 8},
+    {1500, 2, 128, kStaged, 12},    {768, 5, 96, kStaged, 8},       {600, kAny, 64, kStaged, 8},
+    {1024, kAny, 128, kStaged, 8},  {1500, kAny, 128, kStaged, 12}, {kNodeSwapMaxN, kAny, 256, kGlobal, 8},
 };
 constexpr int kNumConfigs = sizeof(kConfigs) / sizeof(kConfigs[0]);
 
@@ -441,7 +628,7 @@ template <int K>
 cudaError_t launch_k(const TwoOptBatch& b, int k, int num_sms, cudaStream_t st) {
     constexpr SwapConfig c = kConfigs[K];
     static_assert(swap_smem(c.max_n, c.threads / 32, c.costs) <= 224 * 1024, "does not fit");
-    if (k == K) return launch_nt<c.threads, c.costs>(b, num_sms, st);
+    if (k == K) return launch_nt<c.threads, c.costs, c.cols>(b, num_sms, st);
     if constexpr (K + 1 < kNumConfigs) return launch_k<K + 1>(b, k, num_sms, st);
     else return cudaErrorInvalidValue;
 }
