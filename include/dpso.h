@@ -241,9 +241,11 @@ int dpso_voxel_occupancy(const double *boxes_dev, int32_t m, const dpso_astar_pa
                          uint8_t *occ_dev, void *stream);
 
 /* n x n int32 A* cost matrix (device, row-major) for n viewpoints (device,
- * n x 3) over the occupancy `occ_dev`.  One thread per pair; each search
- * first gets room for 256 expansions, and pairs that need more are searched
- * again with room for max_expansions.  Synchronises `stream`.  Errors:
+ * n x 3) over the occupancy `occ_dev`.  One warp per pair, its search in shared
+ * memory; searches that outgrow it are made again with more room, at last by
+ * one thread each with room for max_expansions in device memory (grids and
+ * weights beyond the warp's keys: by one thread each from the start, first with
+ * room for 256 expansions).  Synchronises `stream`.  Errors:
  * DPSO_ERR_ARG, DPSO_ERR_RANGE (also: an entry above DPSO_COST_MAX, clamped),
  * DPSO_ERR_NO_MEMORY. */
 int dpso_cost_matrix_astar(const double *xyz_dev, int32_t n, const uint8_t *occ_dev,

@@ -17,8 +17,9 @@
 //    voxels (union-find over the 26-neighbourhood) are blocked without a
 //    search: A* could only exhaust its open list or its cap there.
 //  * Pass 1: one warp per search, its map and open list in shared memory
-//    (astar_warp_kernel); a search that outgrows them is searched again, from
-//    the start, by pass 2: one thread per search with its own binary heap and
+//    (astar_warp_kernel); a search that outgrows them, or is sure to, is
+//    searched from the start with larger ones, of which half as many fit, and
+//    then by pass 2: one thread per search with its own binary heap and
 //    open-addressing map (voxel -> best g, closed; slots stamped by search,
 //    so nothing is cleared) in device scratch, room for the full expansion
 //    cap.  Grids or weights too large for the warp pass's packed keys take
@@ -304,7 +305,7 @@ struct WarpSearch {
     static constexpr int kDistinct = SLOTS - SLOTS / 14;  // inserts before a search hands over
     static constexpr int kBytes = (kSlots + kOpen) * 8;
     static constexpr int kWarps = 224 * 1024 / kBytes;
-    static constexpr int kBits = SLOTS == 2048 ? 11 : (SLOTS == 1024 ? 10 : 9);
+    static constexpr int kBits = SLOTS == 2048 ? 11 : 10;
     static_assert(1 << kBits == SLOTS, "a power of two");
 };
 
@@ -315,7 +316,8 @@ struct WarpArgs {
     const int* comp;
     const int2* pairs;
     int npairs;
-    const unsigned* count;  // when set, *count pairs instead of npairs
+    const int* again;       // when set, the numbers of the pairs to search
+    const unsigned* count;  // ... and how many
     unsigned* queue;  // next pair (zero on entry)
     int a1, a2, a3;
     long long unit_mm;
@@ -342,6 +344,18 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long v)
     return (static_cast<unsigned long long>(mhi) << 32) | mlo;
 }
 
+// About the distinct voxels that a search meets on a free way from s to t: a step
+// along one, two or three axes brings 9, 15 or 19 of the 27 around a voxel into
+// view (in a grid of one or two layers that share of those there are).
+__device__ __forceinline__ int free_way_voxels(const AstarGrid& gr, int s, int t) {
+    const int nxy = gr.nx * gr.ny;
+    const int dx = abs(s % gr.nx - t % gr.nx), dy = abs(s / gr.nx % gr.ny - t / gr.nx % gr.ny),
+              dz = abs(s / nxy - t / nxy);
+    const int top = max(dx, max(dy, dz)), low = min(dx, min(dy, dz)), mid = dx + dy + dz - top - low;
+    return (9 * (top - mid) + 15 * (mid - low) + 19 * low) * min(gr.nx, 3) * min(gr.ny, 3) *
+           min(gr.nz, 3) / 27;
+}
+
 template <int SLOTS>
 __global__ void __launch_bounds__(32 * WarpSearch<SLOTS>::kWarps) astar_warp_kernel(WarpArgs A) {
     using W = WarpSearch<SLOTS>;
@@ -364,11 +378,17 @@ __global__ void __launch_bounds__(32 * WarpSearch<SLOTS>::kWarps) astar_warp_ker
         if (lane == 0) k = static_cast<int>(atomicAdd(A.queue, 1u));
         k = __shfl_sync(0xffffffffu, k, 0);
         if (k >= npairs) break;
+        if (A.again) k = A.again[k];
         const int2 pr = A.pairs[k];
         const int s = A.vox[pr.x], t = A.vox[pr.y];
         long long result = -1;
-        bool handover = false;
-        if (s >= 0 && t >= 0 && A.comp[s] == A.comp[t]) {
+        // A search that the small map cannot hold even on a free way is not
+        // begun there (bridge of 1992 viewpoints, 0.5 m voxels, whole call: 258
+        // ms with the large maps alone, 286 when every search begins in a small
+        // one, 248 so).
+        bool handover = SLOTS == kSmall && s >= 0 && t >= 0 &&
+                        free_way_voxels(A.gr, s, t) + 26 > W::kDistinct;
+        if (!handover && s >= 0 && t >= 0 && A.comp[s] == A.comp[t]) {
             for (int i = lane; i < W::kSlots; i += 32) map[i] = kEmptySlot;
             const int tx = t % nx, ty = (t / nx) % ny, tz = t / nxy;
             const int sx = s % nx, sy = (s / nx) % ny, sz = s / nxy;
@@ -481,9 +501,8 @@ __global__ void __launch_bounds__(32 * WarpSearch<SLOTS>::kWarps) astar_warp_ker
             }
         }
         if (lane == 0) {
-            if (handover) {
-                A.retry[k] = 1;
-            } else {
+            if (SLOTS > kSmall || handover) A.retry[k] = handover;
+            if (!handover) {
                 long long cost = result < 0 ? A.blocked_cost : result * A.unit_mm;
                 if (cost > DPSO_COST_MAX) {
                     atomicOr(A.err, 2);
@@ -560,16 +579,41 @@ __global__ void pairs_kernel(int n, int2* __restrict__ pairs) {
         pairs[first + j - i - 1] = make_int2(i, j);
 }
 
-// Counts the pairs flagged for a second search into *count, and lists them
-// (in whatever order) when `list` is given.
-__global__ void retry_kernel(const int* __restrict__ retry, const int2* __restrict__ pairs,
-                             long long np, unsigned* count, int2* __restrict__ list) {
+// Counts the pairs flagged for a second search into *count, and lists their
+// numbers (in whatever order) when `list` is given.
+__global__ void retry_kernel(const int* __restrict__ retry, long long np, unsigned* count,
+                             int* __restrict__ list) {
     for (long long k = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; k < np;
          k += static_cast<long long>(gridDim.x) * blockDim.x)
         if (retry[k]) {
             const unsigned at = atomicAdd(count, 1u);
-            if (list) list[at] = pairs[k];
+            if (list) list[at] = static_cast<int>(k);
         }
+}
+
+// The flagged pairs in the order of their numbers, by one block: the thread
+// pass runs neighbours of the list in step, and neighbours in row order search
+// much the same way (grid of 400 viewpoints, 0.25 m voxels, whole call: 121 ms;
+// in the order in which the flags were met 137).
+__global__ void __launch_bounds__(1024) ordered_retry_kernel(const int* __restrict__ retry,
+                                                             const int2* __restrict__ pairs,
+                                                             long long np, int2* __restrict__ list) {
+    __shared__ int upto[2][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long at = 0;
+    int par = 0;
+    for (long long k0 = 0; k0 < np; k0 += 1024, par ^= 1) {
+        const long long k = k0 + threadIdx.x;
+        const bool flag = k < np && retry[k];
+        const unsigned mask = __ballot_sync(0xffffffffu, flag);
+        if (lane == 0) upto[par][warp] = __popc(mask);
+        __syncthreads();
+        const int mine = upto[par][lane];  // (every warp sums all warps' counts)
+        const int before = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0);
+        const int all = __reduce_add_sync(0xffffffffu, mine);
+        if (flag) list[at + before + __popc(mask & ((1u << lane) - 1))] = pairs[k];
+        at += all;
+    }
 }
 
 __global__ void zero_diagonal_kernel(int* C, int n) {
@@ -724,7 +768,7 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     };
     const size_t oHead = place(4 * sizeof(int)), oVox = place(sizeof(int) * n),
                  oComp = place(sizeof(int) * nv), oPairs = place(sizeof(int2) * np),
-                 oRetry = place(sizeof(int) * np), oMore = place(sizeof(int2) * np);
+                 oRetry = place(sizeof(int) * np), oMore = place(sizeof(int) * np);
     Scratch scratch, more;  // (each waits for the stream before it is released)
     if (scratch.acquire(at, s) != cudaSuccess) return DPSO_ERR_NO_MEMORY;
     unsigned char* const base = static_cast<unsigned char*>(scratch.p);
@@ -733,7 +777,7 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     unsigned* const again = reinterpret_cast<unsigned*>(err + 3);
     int* const vox = reinterpret_cast<int*>(base + oVox);
     int* const comp = reinterpret_cast<int*>(base + oComp);
-    int2* dpairs = reinterpret_cast<int2*>(base + oPairs);
+    int2* const dpairs = reinterpret_cast<int2*>(base + oPairs);
     int* const retry = reinterpret_cast<int*>(base + oRetry);
     const AstarGrid gr = grid_of(ap);
     cudaError_t e = np > 0 ? cudaMemsetAsync(retry, 0, sizeof(int) * np, s) : cudaSuccess;
@@ -776,7 +820,9 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     if (warp_pass_fits(ap)) {
         // pass 1: every pair, one warp per search in shared memory, the full
         // cap; searches that outgrow the warp's map or open array are searched
-        // again with larger ones, then in pass 2
+        // again with larger ones, then in pass 2.  Pairs that fit one wave of
+        // the large maps start there: the launches between cost more than the
+        // first wave's searches (30 viewpoints, whole call: 340 -> 309 us).
         WarpArgs W{};
         W.gr = gr;
         W.occ = occ_dev;
@@ -797,20 +843,26 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
         A.final_pass = false;
         if (e == cudaSuccess && np > 0) {
             W.queue = queue;
-            e = run_warp_pass<kSmall>(W, s);
-            // the searches that outgrew the small map, with the large one
-            int2* const list = reinterpret_cast<int2*>(base + oMore);
-            if (e == cudaSuccess) {
-                retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, dpairs, np, again, list);
-                e = cudaGetLastError();
+            int dev = 0, sms = 0;
+            e = cudaGetDevice(&dev);
+            if (e == cudaSuccess)
+                e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (np > static_cast<long long>(sms) * WarpSearch<2048>::kWarps) {
+                if (e == cudaSuccess) e = run_warp_pass<kSmall>(W, s);
+                // the searches that outgrew the small map, with the large one
+                int* const list = reinterpret_cast<int*>(base + oMore);
+                if (e == cudaSuccess) {
+                    retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, np, again, list);
+                    e = cudaGetLastError();
+                }
+                W.again = list;
+                W.count = again;
+                W.queue = queue + 1;
+                if (e == cudaSuccess) e = run_warp_pass<2048>(W, s);
+                if (e == cudaSuccess) e = cudaMemsetAsync(again, 0, sizeof(unsigned), s);
+            } else if (e == cudaSuccess) {
+                e = run_warp_pass<2048>(W, s);
             }
-            if (e == cudaSuccess) e = cudaMemsetAsync(retry, 0, sizeof(int) * np, s);
-            W.pairs = list;
-            W.count = again;
-            W.queue = queue + 1;
-            if (e == cudaSuccess) e = run_warp_pass<2048>(W, s);
-            if (e == cudaSuccess) e = cudaMemsetAsync(again, 0, sizeof(unsigned), s);
-            dpairs = list;
         }
     } else {
         // pass 1: every pair, room for a short search
@@ -824,7 +876,7 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
     // pass 2: the pairs that need more room, searched again from the start
     if (e == cudaSuccess && np > 0 && !A.final_pass) {
         unsigned count = 0;
-        retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, dpairs, np, again, nullptr);
+        retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, np, again, nullptr);
         e = cudaGetLastError();
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&count, again, sizeof(count), cudaMemcpyDeviceToHost, s);
@@ -832,9 +884,8 @@ int dpso_cost_matrix_astar(const double* xyz_dev, int32_t n, const uint8_t* occ_
         if (e == cudaSuccess && count > 0) {
             e = more.acquire(sizeof(int2) * count, s);
             int2* const list = static_cast<int2*>(more.p);
-            if (e == cudaSuccess) e = cudaMemsetAsync(again, 0, sizeof(unsigned), s);
             if (e == cudaSuccess) {
-                retry_kernel<<<retry_blocks, 256, 0, s>>>(retry, dpairs, np, again, list);
+                ordered_retry_kernel<<<1, 1024, 0, s>>>(retry, dpairs, np, list);
                 e = cudaGetLastError();
             }
             A.max_exp = ap->max_expansions;
