@@ -42,8 +42,16 @@
 // With T = 0 and no candidate that fits, the tour is 2-optimal.
 //
 // A list that runs full folds its upper part back into low (T falls).  Where
-// more candidates than it holds tie on one delta, so that T cannot rise, a
-// pass scans every row with low < 0 and takes the best directly.
+// more candidates than it holds tie on one delta, so that T cannot rise, passes
+// take the best move directly: they look at the edges in tour order, each
+// against the later ones, and end with the first that attains the smallest low,
+// since of equal deltas the smallest position counts.  The edges before it stay
+// without such a pair but for the edges that the move turns round, so the next
+// pass looks at those alone there.  T is tried again once such passes have
+// looked at eight times the edges that a trial scans.  Costs of 1 and 2, whole
+// call: 300 viewpoints, 1024 tours 12.4 ms when every pass scanned every row,
+// 2.6 so; 700 viewpoints, 300 tours 69 and 9.0; 1500 viewpoints, 48 tours 303
+// and 45.
 //
 // What bounds it: for long tours the gathers of the rows that are scanned in
 // full (the cost rows of the edge's two ends, staged interleaved in shared
@@ -233,7 +241,8 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
         long long scans = 0;  // rows decided: new edges, and rows scanned
         int moves = 0, passes = 0;
         int T = INT_MIN;      // the list holds every candidate with delta < T
-        int direct = 0;       // passes to take directly (ties overflow the list)
+        int clean = 0, clean_lo = 0, clean_moves = -2, last_bi = 0, last_bj = 0;  // direct passes
+        int direct = 0;       // edges that direct passes may still look at (ties overflow the list)
         int level = 0;        // doublings of the groups that choose T' (after a full list)
         int par = 0;
         const int guard = 1000 + 100 * n;
@@ -353,6 +362,41 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
             __syncthreads();
         };
 
+        // The best move over all pairs, which is known to be no better than lo: a
+        // warp per tour position i against the later ones, in order, until one
+        // attains lo.  Of the positions below `clean` only pairs with a j in
+        // [seg_lo, seg_hi] may.  Adds the positions looked at to `looked`.
+        auto direct_best = [&](int lo, int clean, int seg_lo, int seg_hi, int& looked) {
+            const unsigned bound = static_cast<unsigned>(lo) ^ 0x80000000u;
+            unsigned long long found = ~0ull;
+            for (int i0 = 0; i0 < n - 2 && static_cast<unsigned>(found >> 32) > bound;) {
+                const bool part = i0 < clean;  // (a block's share of these is taken at once)
+                const int i1 = part ? min(i0 + 4 * kW, clean) : min(i0 + kW, n - 2);
+                unsigned long long mine = ~0ull;
+                for (int i = i0 + warp; i < i1; i += kW) {
+                    const unsigned ai = at[i], vi = ends[ai & 0x7fff];
+                    const int de = len[ai & 0x7fff];
+                    const int u = ai >> 15 ? vi >> 16 : vi & 0xffff, w = ai >> 15 ? vi & 0xffff : vi >> 16;
+                    const int* const ru = kFull ? mat + u * mld : C + static_cast<size_t>(u) * ldc;
+                    const int* const rw = kFull ? mat + w * mld : C + static_cast<size_t>(w) * ldc;
+                    const int j0 = part ? max(i + 2, seg_lo) : i + 2;
+                    const int j1 = part ? seg_hi + 1 : n;
+#pragma unroll 4
+                    for (int j = j0 + lane; j < j1; j += 32) {
+                        const unsigned aj = at[j], vj = ends[aj & 0x7fff];
+                        const int c0 = aj >> 15 ? vj >> 16 : vj & 0xffff;
+                        const int c1 = aj >> 15 ? vj & 0xffff : vj >> 16;
+                        const int d = ru[c0] + rw[c1] - de - len[aj & 0x7fff];
+                        if (d < 0 && (i > 0 || j < n - 1)) mine = min(mine, pack_key(d, i, j));
+                    }
+                }
+                looked += i1 - i0;
+                i0 = i1;
+                found = min(found, block_best(mine));
+            }
+            return found;
+        };
+
         unsigned long long best = ~0ull;  // the pass's best move
         for (;;) {
             if (max_moves > 0 && moves >= max_moves) break;
@@ -393,10 +437,28 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                     T = 0;
                     break;
                 }
+                if (direct > 0) {
+                    // (after one move since the last direct pass at this lo, the
+                    // positions below that pass's and the move's hold no pair of
+                    // lo but with an edge that the move turned or brought in; where
+                    // none is found at all, what else those hold counts as well)
+                    int looked = 0;
+                    for (int c = clean_lo == lo && moves == clean_moves + 1 ? clean : 0;; c = 0) {
+                        best = direct_best(lo, c, last_bi, last_bj, looked);
+                        if (c == 0 || static_cast<int>(static_cast<uint32_t>(best >> 32) ^ 0x80000000u) == lo)
+                            break;
+                    }
+                    direct -= looked;
+                    scans += looked;
+                    if (best == ~0ull) T = 0;  // every pair was looked at
+                    clean_lo = lo;
+                    clean_moves = moves;
+                    clean = static_cast<int>(best >> 16) & 0xffff;
+                    break;
+                }
                 const int c0 = s_cnt;
-                const bool dir = direct > 0;
                 if ((kGroup << level) > (kW > 1 ? 32 : 16)) hi = lo;
-                int Tn = dir ? 0 : min(0, max(hi, lo + 1));
+                int Tn = min(0, max(hi, lo + 1));
                 // Rows to scan.  A short row's pairs all show in the neighbour
                 // lists of its two ends: a pair that is in neither costs at
                 // least the two radii, so its delta is no less than
@@ -413,12 +475,11 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                     const bool wide = reach(ends[s], len[s]) - 2 * len[s] < Tn;
                     const int k = atomicAdd(wide ? &s_wide : &s_rows, 1);
                     rows[wide ? n - 1 - k : k] = static_cast<uint16_t>(s);
-                    if (!dir) low[s] = INT_MAX;
+                    low[s] = INT_MAX;
                 }
                 __syncthreads();
                 const int ns = s_rows, nr = s_wide;
                 const uint16_t* const wrows = rows + n - nr;  // (in whatever order)
-                unsigned long long mine = ~0ull;
                 // Scans the pairs that edge e (staged in buffer k) owns, over
                 // slots t0, t0 + step, ..: candidates in [T, Tn) go to the list,
                 // the smallest delta past Tn is returned.
@@ -448,15 +509,10 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
 #pragma unroll
                             for (int q = 0; q < kBatch; ++q) {
                                 const int s = s0 + q * step;
-                                if (dir) {
-                                    if (d0[q] < 0) mine = min(mine, key_of(d0[q], e, s, 0));
-                                    if (d1[q] < 0) mine = min(mine, key_of(d1[q], e, s, 1));
-                                } else {
-                                    if (d0[q] >= T && d0[q] < Tn) insert(d0[q], e, s, 0);
-                                    if (d1[q] >= T && d1[q] < Tn) insert(d1[q], e, s, 1);
-                                    if (d0[q] >= Tn) m = min(m, d0[q]);
-                                    if (d1[q] >= Tn) m = min(m, d1[q]);
-                                }
+                                if (d0[q] >= T && d0[q] < Tn) insert(d0[q], e, s, 0);
+                                if (d1[q] >= T && d1[q] < Tn) insert(d1[q], e, s, 1);
+                                if (d0[q] >= Tn) m = min(m, d0[q]);
+                                if (d1[q] >= Tn) m = min(m, d1[q]);
                             }
                         }
                         lbe = min(lbe, m);
@@ -518,13 +574,12 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                             const int s = slot[k] & 0x1fff, d = nb[k / 2].x + c2[k] - de - len[s];
                             const int type = (slot[k] >> 13) == (side == 0 ? 1 : 0) ? 0 : 1;
                             if (d >= Tn) lbe = min(lbe, d);
-                            else if (dir) mine = min(mine, d < 0 ? key_of(d, e, s, type) : ~0ull);
                             else if (d >= T) insert(d, e, s, type);
                         }
 #pragma unroll
                         for (int o = 1; o < 8; o <<= 1)
                             lbe = min(lbe, __shfl_xor_sync(0xffffffffu, lbe, o));
-                        if (on && !dir && (lane & 7) == 0 && lbe < 0) atomicMin(&low[e], lbe);
+                        if (on && (lane & 7) == 0 && lbe < 0) atomicMin(&low[e], lbe);
                     }
                 };
                 bool shrunk = false;
@@ -543,7 +598,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                             __syncwarp();
                             const int e = wrows[r];
                             const int lbe = scan(k, e, lane, 32);
-                            if (!dir && lane == 0) atomicMin(&low[e], lbe);
+                            if (lane == 0) atomicMin(&low[e], lbe);
                             __syncwarp();  // the buffer is no longer read
                         }
                         if (kStages) cp_wait_all();
@@ -557,7 +612,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                             if (r + 1 < nr) load_row(k ^ 1, r + 1, tid, NT);
                             const int e = wrows[r];
                             const int lbe = scan(k, e, tid, NT);
-                            if (!dir && lane == 0) atomicMin(&low[e], lbe);
+                            if (lane == 0) atomicMin(&low[e], lbe);
                         }
                     }
                     __syncthreads();
@@ -565,8 +620,8 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                     // The list ran full: T' falls to the largest, over 32 groups of
                     // threads, of the group's smallest delta, what this round
                     // added is dropped and its rows are scanned again.  Where T'
-                    // cannot stay above T (ties), T falls too and the next
-                    // passes are direct.
+                    // cannot stay above T (ties), T falls too, which bounds those
+                    // rows as well, and the next passes are direct.
                     int mk = INT_MAX;
                     for (int k = tid; k < cap; k += NT)
                         if (list[k] != kDead) mk = min(mk, static_cast<int>(list[k] >> 32));
@@ -581,23 +636,21 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                     for (int w = 1; w < kW; ++w) t = max(t, s_hi[w]);
                     Tn = min(Tn, t);
                     fold(Tn, T);
+                    shrunk = true;
                     if (Tn <= T) {
                         T = Tn;
-                        direct = 16;
+                        direct = 8 * n;
+                        for (int k = tid; k < ns + nr; k += NT)
+                            low[k < ns ? rows[k] : wrows[k - ns]] = T;
+                        __syncthreads();
+                        break;
                     }
-                    shrunk = true;
                 }
                 const int cnt = s_cnt;
-                if (!dir) mine = list_best(min(c0, cnt), cnt);
-                best = block_best(mine);
-                if (dir) {
-                    --direct;
-                    if (best == ~0ull) T = 0;  // every row was looked at
-                } else {
-                    T = Tn;
-                    if (shrunk) level = min(level + 1, 6);
-                    else if (level > 0 && cnt < cap / 4) --level;
-                }
+                best = block_best(list_best(min(c0, cnt), cnt));
+                T = Tn;
+                if (shrunk) level = min(level + 1, 6);
+                else if (level > 0 && cnt < cap / 4) --level;
             }
             ++passes;
             if (best == ~0ull) break;
@@ -606,6 +659,8 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
             const int bi = static_cast<int>((best >> 16) & 0xffffu);
             const int bj = static_cast<int>(best & 0xffffu);
             f += static_cast<int>(static_cast<uint32_t>(best >> 32) ^ 0x80000000u);
+            last_bi = bi;
+            last_bj = bj;
             const unsigned ae = at[bi], ah = at[bj];
             const int e = ae & 0x7fff, h = ah & 0x7fff;
             const unsigned ve = ends[e], vh = ends[h];
