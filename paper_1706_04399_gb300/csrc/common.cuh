@@ -286,7 +286,7 @@ int node_swap_class(int n);  // launch configuration: members that agree share a
 cudaError_t launch_node_swap(const TwoOptBatch& b, int num_sms, cudaStream_t st);
 
 // ---- scratch.cu ----
-constexpr size_t kScratchSlotBytes = 128 * 1024;
+constexpr size_t kScratchSlotBytes = 1024 * 1024;
 // Device scratch of one synchronous call.  The call waits for its stream
 // before it releases the scratch (the destructor does on every path).
 struct Scratch {
@@ -294,6 +294,8 @@ struct Scratch {
     cudaStream_t stream = nullptr;
     int device = 0, slot = -1;
     cudaError_t acquire(size_t bytes, cudaStream_t st);
+    // One of the fixed slots or nothing (p stays null): never allocates.
+    cudaError_t acquire_slot(size_t bytes, cudaStream_t st);
     void release();
     Scratch() = default;
     Scratch(const Scratch&) = delete;

@@ -6,8 +6,9 @@
 // A slot is held from acquire to release by one call, which has waited for its
 // stream in between, so calls on any streams and host threads have slots of
 // their own; when all are taken, or the call needs more than a slot, it
-// allocates as before.  Every GPU that loads the library holds the slots (1
-// MiB) until the process exits.
+// allocates as before.  A slot holds the 2-opt's neighbour lists for tours of up
+// to 4000 viewpoints.  Every GPU that loads the library holds the slots (8 MiB)
+// until the process exits.
 #include <atomic>
 
 #include "common.cuh"
@@ -21,26 +22,30 @@ std::atomic<unsigned> g_taken[kMaxDevices];  // bit per slot, by device
 
 }  // namespace
 
-cudaError_t Scratch::acquire(size_t bytes, cudaStream_t st) {
+cudaError_t Scratch::acquire_slot(size_t bytes, cudaStream_t st) {
     stream = st;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (bytes <= kScratchSlotBytes && dev < kMaxDevices) {
-        for (int k = 0; k < kSlots; ++k) {
-            if (g_taken[dev].fetch_or(1u << k, std::memory_order_acquire) >> k & 1) continue;
-            void* base = nullptr;
-            e = cudaGetSymbolAddress(&base, g_slots);
-            if (e != cudaSuccess) {
-                g_taken[dev].fetch_and(~(1u << k), std::memory_order_release);
-                return e;
-            }
-            device = dev;
-            slot = k;
-            p = static_cast<unsigned char*>(base) + k * kScratchSlotBytes;
-            return cudaSuccess;
+    if (e != cudaSuccess || bytes > kScratchSlotBytes || dev >= kMaxDevices) return e;
+    for (int k = 0; k < kSlots; ++k) {
+        if (g_taken[dev].fetch_or(1u << k, std::memory_order_acquire) >> k & 1) continue;
+        void* base = nullptr;
+        e = cudaGetSymbolAddress(&base, g_slots);
+        if (e != cudaSuccess) {
+            g_taken[dev].fetch_and(~(1u << k), std::memory_order_release);
+            return e;
         }
+        device = dev;
+        slot = k;
+        p = static_cast<unsigned char*>(base) + k * kScratchSlotBytes;
+        break;
     }
+    return cudaSuccess;
+}
+
+cudaError_t Scratch::acquire(size_t bytes, cudaStream_t st) {
+    cudaError_t e = acquire_slot(bytes, st);
+    if (e != cudaSuccess || p) return e;
     e = cudaMallocAsync(&p, bytes, st);
     if (e != cudaSuccess) {
         cudaGetLastError();

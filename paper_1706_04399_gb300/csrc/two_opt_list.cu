@@ -26,11 +26,18 @@
 //  * A pair belongs to its longer edge (ties: the larger slot).  low[slot] is
 //    a lower bound on the deltas of the slot's own pairs that are not in the
 //    list; before anything is known it is -2 C[u][w], since a pair's delta is
-//    no smaller than minus its edges.  When no candidate fits, T is raised to
+//    no smaller than minus its edges (with neighbour lists, below, the cheapest
+//    neighbours of u and w are added).  When no candidate fits, T is raised to
 //    T' and the slots with low < T' scan their row: candidates in [T, T') go
 //    to the list, the smallest delta past T' becomes the slot's low.
 //  * T' is the largest, over groups of threads, of the group's smallest low:
-//    about G ln G rows for G groups, a few scans per move in all.
+//    about G ln G rows for G groups, a few scans per move in all.  From the
+//    fifth raise in a row on, every one that brings no move is made with twice
+//    as many groups: a tour that is 2-optimal already needs all its rows, and
+//    would take some 20 of them at a time (1200 viewpoints, 48 such tours, whole
+//    call: 72 raises and 600 us, now 255, of which 190 were an allocation; with
+//    doubling from the second raise the first moves of random tours scan too
+//    much, 150 tours, one move: 137 -> 766 us).
 // Longer tours (kLists) also save on those scans:
 //  * Every city has a list of its 32 cheapest neighbours.  A pair that shows in
 //    neither list of an edge's two ends costs at least the lists' radii there,
@@ -227,7 +234,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
             const int d = C[static_cast<size_t>(u) * ldc + w];
             ends[i] = u | (w << 16);
             len[i] = d;
-            low[i] = -2 * d;
+            low[i] = -2 * d + (near ? near[u * kNear].x + near[w * kNear].x : 0);
             inc[u] = i | ((i == 0 ? n - 1 : i - 1) << 16);
             pos[i] = static_cast<uint16_t>(i);
             at[i] = static_cast<uint16_t>(i);
@@ -418,7 +425,8 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
 #pragma unroll 4
                 for (int s = tid; s < n; s += NT) mn = min(mn, low[s]);
                 int gm = mn;
-                for (int o = 1; o < min(kGroup << level, 32); o <<= 1)
+                const int group = (kGroup << level) >> min(max(rounds - 3, 0), 5);
+                for (int o = 1; o < min(group, 32); o <<= 1)
                     gm = min(gm, __shfl_xor_sync(0xffffffffu, gm, o));
                 mn = __reduce_min_sync(0xffffffffu, mn);
                 gm = __reduce_max_sync(0xffffffffu, gm == INT_MAX ? INT_MIN : gm);
@@ -457,7 +465,7 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
                     break;
                 }
                 const int c0 = s_cnt;
-                if ((kGroup << level) > (kW > 1 ? 32 : 16)) hi = lo;
+                if (group > (kW > 1 ? 32 : 16)) hi = lo;
                 int Tn = min(0, max(hi, lo + 1));
                 // Rows to scan.  A short row's pairs all show in the neighbour
                 // lists of its two ends: a pair that is in neither costs at

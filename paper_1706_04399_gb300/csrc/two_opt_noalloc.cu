@@ -1,6 +1,7 @@
 // dpso_two_opt_noalloc: the standalone 2-opt entry point without any device
 // allocation.  Its scratch (error word, work queue, totals and per-tour pass /
-// move counts) lives in one fixed array inside the library.  It runs the list
+// move counts) lives in one fixed array inside the library, neighbour lists that
+// do not fit there in one of its fixed scratch slots.  It runs the list
 // kernel of dpso_two_opt, which reads the caller's cost matrix as it is.
 //
 // Who needs it: callers that must not allocate device memory while they run,
@@ -121,12 +122,20 @@ extern "C" int dpso_two_opt_noalloc(const int32_t* C_dev, int32_t n, uint16_t* t
     a.status = err;
     a.tour_passes = scratch + kHeaderWords;
     a.tour_moves = scratch + kHeaderWords + count;
-    // neighbour lists in what the counts leave of the array, when they fit
-    // (without them the kernel scans whole rows)
+    // neighbour lists in what the counts leave of the array, or in one of the
+    // library's fixed scratch slots, when they fit (without them the kernel
+    // scans whole rows)
     const size_t lists_at = (used + 15) / 16 * 16;
-    if (near_used(n, count, sms) && lists_at + near_bytes(n) <= kScratchBytes) {
-        int2* near = reinterpret_cast<int2*>(reinterpret_cast<char*>(scratch) + lists_at);
-        if (e == cudaSuccess) e = build_near(C_dev, n, n, near, st);
+    Scratch slot;
+    if (near_used(n, count, sms)) {
+        int2* near = nullptr;
+        if (lists_at + near_bytes(n) <= kScratchBytes) {
+            near = reinterpret_cast<int2*>(reinterpret_cast<char*>(scratch) + lists_at);
+        } else if (e == cudaSuccess) {
+            e = slot.acquire_slot(near_bytes(n), st);
+            near = static_cast<int2*>(slot.p);
+        }
+        if (e == cudaSuccess && near) e = build_near(C_dev, n, n, near, st);
         a.near = near;
     }
     TwoOptTask* task = reinterpret_cast<TwoOptTask*>(scratch + kTaskWord);
@@ -147,6 +156,7 @@ extern "C" int dpso_two_opt_noalloc(const int32_t* C_dev, int32_t n, uint16_t* t
         e = cudaMemcpyAsync(header, scratch, sizeof(header), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return DPSO_ERR_CUDA;
+    slot.release();  // (the stream was waited for)
     if (static_cast<int>(header[0]) == DPSO_ERR_INTERNAL) return DPSO_ERR_INTERNAL;
     unsigned long long pairs = header[2] | (static_cast<unsigned long long>(header[3]) << 32);
     unsigned long long moves = header[4] | (static_cast<unsigned long long>(header[5]) << 32);
