@@ -55,12 +55,14 @@ __device__ __forceinline__ long long tour_cost_warp(const int* __restrict__ C, i
 // SMs uneven (4096 tours: four blocks on some, three on the others).  One warp
 // per tour in blocks of eight, then now, random tours: 4096 x 1992 39.2 -> 35.0
 // us, 512 x 1992 18.6 -> 10.4, 64 x 2999 26.0 -> 8.5, 1 x 2999 11.2 -> 6.2.
-__global__ void fitness_kernel(const int* __restrict__ C, int ldc, int n,
+template <bool SPLIT>
+__global__ void __launch_bounds__(256) fitness_kernel(const int* __restrict__ C, int ldc, int n,
                                const uint16_t* __restrict__ tours, int ldt, int count,
-                               long long* __restrict__ out, int split) {
+                               long long* __restrict__ out, int log_split) {
     __shared__ long long part[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int w = (blockIdx.x * (blockDim.x >> 5) + warp) / split, sub = warp % split;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, split = SPLIT ? 1 << log_split : 1;
+    const int w = (blockIdx.x * (blockDim.x >> 5) + warp) >> (SPLIT ? log_split : 0);
+    const int sub = SPLIT ? warp & (split - 1) : 0;
     long long f = 0;
     if (w < count) {
         const uint16_t* x = tours + (size_t)w * ldt;
@@ -81,7 +83,7 @@ __global__ void fitness_kernel(const int* __restrict__ C, int ldc, int n,
         }
     }
     f = warp_sum(f);
-    if (split > 1) {  // (the same for the whole grid)
+    if (SPLIT) {
         if (lane == 0) part[warp] = f;
         __syncthreads();
         for (int q = 1; sub == 0 && q < split; ++q) f += part[warp + q];
@@ -635,21 +637,28 @@ int move_warps(const BatchView& b) {
 cudaError_t launch_fitness(const int* C, int ldc, int n, const uint16_t* tours, int ldt, int count,
                            long long* out, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    int split = 1;
+    int log_split = 0;
     // A tour of one round is not split, and eight of them share a block (4096
-    // tours of 64: 5.5 us, in blocks of two 5.8).
+    // tours of 64: 5.5 us, in blocks of two 5.8); so do tours of two rounds, and
+    // tours enough for eight blocks of eight per SM, where the number of blocks
+    // counts more than uneven SMs (60000 tours of 257: 45.7 us in blocks of two,
+    // 37.2 in blocks of eight).  Where C does not fit L2 and there are tours
+    // enough to fill the chip, splitting loses a little (1000 tours of 8192: 110
+    // us whole, 117 split; 300 tours 72 and 40).
     int threads = 256;
     if (n > 256) {
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        while (split < 8 && 256 * split < n && 2ll * split * count <= 64 * sms) split *= 2;
-        threads = max(64, 32 * split);
+        while (log_split < 3 && (256 << log_split) < n &&
+               (2ll << log_split) * count <= 64 * sms)
+            ++log_split;
+        if (log_split > 0 || (n > 512 && count < 64 * sms)) threads = max(64, 32 << log_split);
     }
-    const int per = threads / (32 * split);
-    fitness_kernel<<<(count + per - 1) / per, threads, 0, st>>>(C, ldc, n, tours, ldt, count, out,
-                                                               split);
+    const int per = threads / (32 << log_split);
+    auto* kern = log_split > 0 ? fitness_kernel<true> : fitness_kernel<false>;
+    kern<<<(count + per - 1) / per, threads, 0, st>>>(C, ldc, n, tours, ldt, count, out, log_split);
     return cudaGetLastError();
 }
 
