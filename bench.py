@@ -15,18 +15,18 @@ value   particle-iterations/s = particles x generations / device time of the
         matrix and swarm resident in HBM; the L2 is flushed between timed
         generations.  For N > 1 each rank runs an independent replica (the
         solver has no exchange step to shard).
-2-opt moves/s  candidate 2-opt pairs the exchange kernel decided (evaluated, or
-        excluded by a bound on their row) per second of its own device time
-        (`two_opt_pairs_evaluated_per_s`); the pairs a plain best-improvement
-        scan of the same passes would take are reported beside it.
+2-opt moves/s  candidate 2-opt pairs the exchange kernel decided per second of its
+        own device time (`two_opt_pairs_decided_per_s`): evaluated, or excluded
+        by a bound on their row without being read, so it is no rate of
+        evaluations; the pairs a plain best-improvement scan of the same passes
+        would take, and the moves applied, are reported beside it.
 e2e     the same metric through dpso_plan from pinned host buffers: copies in,
         cost matrix, initialisation, `steps` generations, best tour out.
-roofline  the 2-opt kernel: 8 bytes of C per candidate pair decided (two int32
-        entries, which an excluded pair does not read) over its CUDA-event time
-        inside the timed generations, against the L2 read bandwidth measured in
-        this run (the cost matrix is L2-resident).  The node-swap kernel counts
-        the plain scan's pairs, nearly all of which it need not look at, so it
-        has no such figure.
+roofline  the exchange kernel: its CUDA-event time inside the timed generations
+        and the L2 read bandwidth measured in this run, without an achieved
+        rate: the kernels read few of the pairs they decide and count no bytes
+        (a capture puts L2 at 5 % of its peak), and what bounds them is the
+        chain of a pass.
 fitness_roofline  the tour-fitness kernel (Eq. min) over the swarm's tours:
         4 n bytes of C gathered per tour over its CUDA-event time, against the
         random 4-byte gather rate from an L2-resident buffer measured in this
@@ -51,8 +51,6 @@ sys.path.insert(0, ROOT)
 
 METRIC = "DPSO particle-iterations/s and 2-opt moves/s per GB300; batched p99 latency"
 UNIT = "particle-iterations/s"
-BYTES_PER_PAIR = 8          # 2-opt: C[x_i][x_j] + C[x_i+1][x_j+1], int32 each
-BYTES_PER_SWAP_PAIR = 16    # node swap: the four new edges' costs, int32 each
 DEFAULT_STEPS = {"bridge": 20, "facade": 100, "tiny": 100, "batched": 3, "astar": 20,
                  "two-opt": 3, "serving": 1}
 
@@ -457,7 +455,7 @@ def gpu_line(args):
     value = job_throughput(S * args.steps, world, dev_ms_max)
 
     pairs = st1["two_opt_pairs"] - st0["two_opt_pairs"]
-    evaluated = st1["two_opt_evaluated"] - st0["two_opt_evaluated"]
+    decided = st1["two_opt_evaluated"] - st0["two_opt_evaluated"]
     moves = st1["two_opt_moves"] - st0["two_opt_moves"]
     two_ms = timing["ms"]["two_opt"]
     launches = sum(timing["launches"].values())
@@ -467,25 +465,17 @@ def gpu_line(args):
         probes = {f"{mb}MiB": dpso.dpso_probe_l2_read_gbs(mb << 20, max(1, 960 // mb))
                   for mb in (8, 16, 24)}
         l2 = max(probes.values())
-        bpp = BYTES_PER_SWAP_PAIR if node_swap else BYTES_PER_PAIR
-        # bytes of the pairs the kernel decided, not of the pairs a plain scan
-        # would take (the node swap reports only the latter: no figure)
-        achieved = bpp * evaluated / (two_ms / 1e3) / 1e9 if two_ms > 0 else 0.0
-        if node_swap:
-            achieved = 0.0
         traffic = None if node_swap else dram_traffic("two_opt_list_kernel", inst.name)
         roofline = {
             "kernel": "node_swap_kernel" if node_swap else "two_opt_list_kernel",
-            "bound": "l2", "bytes_per_pair": bpp, "pairs_evaluated": evaluated,
-            "achieved": achieved, "peak": l2,
-            "unit": "GB/s", "frac": achieved / l2 if l2 else None,
+            "bound": "latency of a pass (no achieved rate: the kernel counts no bytes)",
+            "ms": two_ms, "achieved": None, "peak": l2, "unit": "GB/s", "frac": None,
             "traffic": traffic,
             "peak_source": "L2 read bandwidth measured in this run by dpso_probe_l2_read_gbs "
                            "(16-byte loads of an L2-resident buffer, best of 5 runs, best of "
                            "8/16/24 MiB buffers)",
             "l2_probes_gbs": probes,
             "hbm_peak_gbs": peaks.get("hbm_gbs"),
-            "frac_of_hbm_peak": achieved / peaks["hbm_gbs"] if peaks.get("hbm_gbs") else None,
         }
         fit_roof = fitness_roofline(dpso, C, n, sw.state()["X"], stream, inst.name)
         cpu = None
@@ -534,12 +524,13 @@ def gpu_line(args):
             "vs_baseline": None, "dtype": "i32", "data": "synthetic",
             "config": config,
             # the metric's "2-opt moves/s": candidate pairs the kernel decided
-            "two_opt_pairs_evaluated_per_s": evaluated / (two_ms / 1e3) if two_ms > 0 else 0.0,
-            "two_opt_pairs_evaluated": evaluated,
+            "two_opt_pairs_decided_per_s": decided / (two_ms / 1e3) if two_ms > 0 else 0.0,
+            "two_opt_pairs_decided": decided,
             # what a plain best-improvement scan of the same passes would take
             "two_opt_plain_scan_pairs": pairs,
             "two_opt_plain_scan_pairs_per_s": pairs / (two_ms / 1e3) if two_ms > 0 else 0.0,
             "two_opt_moves_applied": moves,
+            "two_opt_moves_applied_per_s": moves / (two_ms / 1e3) if two_ms > 0 else 0.0,
             "phase_ms": phases, "wall_s": wall,
             "roofline": roofline, "fitness_roofline": fit_roof, "cpu_baseline": cpu, "e2e": e2e,
             "gpu_launches": launches, "clocks": sampler.summary(),
