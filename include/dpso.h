@@ -260,8 +260,8 @@ int dpso_cost_matrix_astar(const double *xyz_dev, int32_t n, const uint8_t *occ_
  * cyclic tour) whose swap shortens the tour most, ties to the smallest
  * (delta, i, j), until no swap improves or `max_moves` (> 0) swaps were made.
  * Arguments, layout and errors as dpso_two_opt, except that entries of C must
- * be at most DPSO_NODE_SWAP_COST_MAX (else DPSO_ERR_RANGE, as for n too large
- * for a shared-memory tile); *pairs_host counts n(n-1)/2 per pass.
+ * be at most DPSO_NODE_SWAP_COST_MAX (else DPSO_ERR_RANGE, as for n > 4497);
+ * *pairs_host counts n(n-1)/2 per pass.
  * Synchronises `stream`.
  */
 int dpso_node_swap(const int32_t *C_dev, int32_t n, uint16_t *tours_dev, int32_t count,
@@ -376,8 +376,8 @@ int dpso_batch_autotune(dpso_batch *b, dpso_two_opt_shape *chosen, void *stream)
 int dpso_batch_set_two_opt_shape(dpso_batch *b, const dpso_two_opt_shape *shape);
 /* The tiled 2-opt kernel's default launch shape for a launch over `count` tours
  * of n viewpoints on a GPU with `num_sms` SMs (a launch implementation choice;
- * the paper has none; unpinned launches run the list kernel instead).  Up to n = 256: 32-row tiles, two tours per
- * CTA; beyond: the shape with the most tile rows in flight per SM, except that
+ * the paper has none; unpinned launches run the list kernel instead).  Up to
+ * n = 256: 32-row tiles, two tours per CTA; beyond: the shape with the most tile rows in flight per SM, except that
  * tours whose tallest fitting tile has 16 rows or fewer take 8-row tiles with
  * two tours per CTA when those fit and count >= 2 * num_sms.  All zero when
  * no tiled shape fits.  Host only, no device call.
@@ -475,7 +475,9 @@ int dpso_server_create(dpso_server **out, const dpso_server_params *p);
 int dpso_server_submit(dpso_server *s, const dpso_request *r, int64_t *id);
 /* The device bytes admission charges for a request (host only, no device
  * needed): the swarm arrays dpso_init allocates for its n, swarm size,
- * generation budget and flags, plus the transient cost-matrix buffers. */
+ * generation budget and flags, for a 2-opt the row-shifted cost copies that a
+ * shape pinned on a batch would add (the server pins none: this keeps the
+ * charge on the safe side), plus the transient cost-matrix buffers. */
 int dpso_server_footprint(const dpso_request *r, uint64_t *bytes);
 /* *state: 0 queued or running, 1 done, or the negative status the request
  * failed with (DPSO_ERR_NO_MEMORY when its footprint exceeds the whole

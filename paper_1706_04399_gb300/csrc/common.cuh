@@ -73,7 +73,7 @@ struct Ctl {
     unsigned long long pairs;  // 2-opt candidate pairs evaluated
     unsigned long long moves;  // 2-opt moves applied
     unsigned long long runs;   // generations with an edge exchange
-    unsigned long long evals;  // candidate pairs the exchange kernels evaluated
+    unsigned long long evals;  // candidate pairs the exchange kernels decided
     long long* hist;           // gbest cost after each generation
     int hist_cap;
     int pad1;
@@ -167,7 +167,7 @@ cudaError_t launch_gbest(const BatchView& b, int second, unsigned int* queue, in
 cudaError_t launch_philox_draws(unsigned long long seed, uint32_t phase, uint32_t iter,
                                 uint32_t particle, int count, uint32_t* out, cudaStream_t st);
 
-// ---- launchers (two_opt_list.cu, two_opt_tiled.cu) ----
+// ---- launchers (two_opt_list.cu) ----
 // One 2-opt problem: best-improvement 2-opt on `count` tours of length n (row
 // stride ldt), updating tours, costs and (when pbest != nullptr) the pbest
 // arrays.  When `gate` is non-null nothing happens unless *gate != 0.
@@ -196,9 +196,9 @@ struct TwoOptTask {
     // on it, only the time the last tour finishes does.
     const int* order;
     int kind;  // exchange neighbourhood: 0 edge exchange (2-opt), 1 node swap
-    // Optional: receives the candidate pairs the kernel actually evaluated
-    // (fewer than *pairs, the pairs a plain best-improvement pass scans, when
-    // the kernel reuses the previous pass's row minima).
+    // Optional: receives the candidate pairs the kernel decided (evaluated, or
+    // excluded by a bound on their row): fewer than *pairs, the pairs a plain
+    // best-improvement pass scans, where it knows from earlier passes.
     unsigned long long* evals;
 };
 
@@ -235,9 +235,6 @@ cudaError_t launch_two_opt_small(const TwoOptBatch& b, int num_sms, cudaStream_t
 // one SM then holds: members that agree share a launch.
 int two_opt_class(int n, int* ctas);
 
-// ---- two_opt_tiled.cu: pipelined tiled variant (needs the shifted copies) ----
-// Row pitch (words) of the shifted copies and of the staged rows: room for a
-// shift of up to 3 words, a multiple of 4 words (16-byte rows), ldq/4 odd.
 // Raises a kernel's dynamic shared-memory limit to the most the device
 // allows beside the kernel's static shared memory, and checks that `smem`
 // bytes fit.  Every caller sets the same value, so launches of one kernel
@@ -257,6 +254,9 @@ inline cudaError_t raise_smem_limit(Kernel* kernel, size_t smem) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max);
 }
 
+// ---- two_opt_tiled.cu: pipelined tiled variant (needs the shifted copies) ----
+// Row pitch (words) of the shifted copies and of the staged rows: room for a
+// shift of up to 3 words, a multiple of 4 words (16-byte rows), ldq/4 odd.
 __host__ __device__ inline int shifted_ld(int n) {
     int q = (n + 3 + 3) / 4 * 4;
     if (((q / 4) & 1) == 0) q += 4;
@@ -273,12 +273,6 @@ bool two_opt_tiled_fits(int n, int rows, int tpc, int tg);  // a valid shape tha
 cudaError_t build_shifted_copies(const int* C, int ldc, int n, int* Cs, cudaStream_t st);
 cudaError_t launch_two_opt_tiled(const TwoOptBatch& b, int rows, int tpc, int tg, int num_sms,
                                  cudaStream_t st);
-// ---- two_opt_list.cu: the default 2-opt kernel, any n ----
-cudaError_t launch_two_opt_list(const TwoOptBatch& b, int num_sms, cudaStream_t st);
-// Launch configuration (a number from 0) for tours of up to n viewpoints, and
-// the tours one SM then holds.
-int two_opt_list_class(int n, int* ctas);
-
 // ---- node_swap.cu: node-swap exchange (entries of C at most
 // DPSO_NODE_SWAP_COST_MAX) ----
 bool node_swap_fits(int n);

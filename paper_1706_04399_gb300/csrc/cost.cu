@@ -107,8 +107,9 @@ __device__ __forceinline__ Split split(double v) {
 }
 
 // 1000 |q - p| rounded to the nearest integer, in pairs of FP32 numbers (sums
-// with their rounding error, products with theirs by FMA), where the result is
-// not near a tie; -1: not decided.  With M the largest coordinate magnitude,
+// with their rounding error after Knuth and, for ordered terms, Dekker, products
+// with theirs by FMA, the root by one Newton correction of the reciprocal square
+// root), where the result is not near a tie; -1: not decided.  With M the largest coordinate magnitude,
 // the differences are off by some 2^-46 M and everything after by some 2^-44
 // of itself, so the length r in mm by less than (r + 1000 M) 2^-40; a tie
 // closer than 2^8 times that (and 2^-20) is left to FP64, whose own error is

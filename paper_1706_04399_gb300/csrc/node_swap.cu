@@ -51,7 +51,7 @@ using namespace tiled;
 // stale position is looked at.  ~0: no improving pair.
 constexpr unsigned long long kExact = 0x8000;
 constexpr unsigned long long kNone = ~0ull;
-constexpr int kNodeSwapMaxN = 4497;  // longer tours are refused
+constexpr int kNodeSwapMaxN = 4497;  // longer tours are refused (as the header says)
 constexpr int kThreadsPerSm = 640;  // the register budget's resident threads
 constexpr int kRowsStaged = 10;  // two swapped positions, two on each side
 
