@@ -917,19 +917,32 @@ cudaError_t launch_cfg(const TwoOptBatch& b, int cap, int num_sms, cudaStream_t 
 
 // Launch configurations: for tours of up to max_n viewpoints (and, with
 // `few`, launches of at most that many tours per SM): threads per tour,
-// staging, list entries.  Measured on GB300 (random grid, facade and bridge
-// tours to 2-optimality, whole call, ms; warp = each warp stages its rows;
-// with four partners in flight and 16 groups):
-//   n     tours  matrix 256  warp 64 / 128  CTA 128 / 256 / 512   C 128 / 256
-//   157   256    0.70        1.02 / 0.80                          0.80 / -
-//   157   1024   1.31        1.25 / 1.43                          1.39 / -
-//   220   128    0.86        -    / 1.07                          1.03 / 0.87
-//   400   256    -           3.13 / 2.30    2.45 / - / -          2.30 / 1.94
-//   400   1024   -           4.12 / 4.65    4.86 / - / -          4.60 / -
-//   1000  150    -           -              5.53 / 4.75 / -       5.67 / 4.15
-//   1000  600    -           -              7.14 / 10.0 / -       7.45 / 9.21
-//   1992  600    -           -              31.1 / 27.6 / 41.7    57.5 / 30.6
-//   2999  150    -           -              -    / 19.4 / 19.3    -    / 24.1
+// staging, list entries.  Measured on GB300 (random tours of a grid, at 1992 of
+// the bridge, to 2-optimality, whole call, ms; warp = each warp stages its rows;
+// CTA and C with neighbour lists):
+//   n     tours  matrix 256  warp 64 / 128  CTA 128 / 256  C 128 / 256
+//   157   256    0.42        0.58 / 0.47    -              0.52 / 0.51
+//   157   1024   1.27        0.74 / 0.95    -              0.95 / 1.60
+//   200   128    0.48        -    / 0.58    -              0.66 / 0.59
+//   220   128    0.49        -    / 0.68    -              0.78 / 0.64
+//   200   304    -           0.80 / 0.64    -              0.72 / 0.67
+//   200   450    -           0.86 / 0.68    -              0.76 / 1.15
+//   400   150    -           1.90 / 1.34    -              1.48 / 1.27
+//   400   304    -           1.91 / 1.56    -              1.64 / 1.43
+//   400   330    -           2.04 / 1.65    -              1.64 / 2.29
+//   400   608    -           2.23 / 2.02    -              1.85 / 2.67
+//   400   1024   -           2.82 / 3.38    -              3.18 / 4.74
+//   512   450    -           2.80 / 2.17    -              2.20 / 3.38
+//   512   1024   -           5.68 / 4.67    -              4.17 / 6.37
+//   700   150    -           -              2.95 / 2.46    2.87 / 2.42
+//   1000  150    -           -              4.63 / 3.81    4.74 / 3.87
+//   1000  304    -           -              4.99 / 4.48    5.22 / 4.56
+//   1000  600    -           -              6.28 / 8.70    6.67 / 8.81
+//   1200  150    -           -              5.89 / 4.98    6.22 / 5.13
+//   1200  600    -           -              8.17 / 11.4    9.29 / 11.8
+//   1992  600    -           -              30.6 / 26.2    -    / 31.6
+//   2999  150    -           -              -    / 18.1    -    / 24.9
+// (512 viewpoints and 64 threads: six tours an SM, so 1024 take two waves.)
 struct ListConfig {
     int max_n, few, threads;
     Staging staging;
