@@ -56,13 +56,13 @@ __device__ __forceinline__ long long tour_cost_warp(const int* __restrict__ C, i
 // per tour in blocks of eight, then now, random tours: 4096 x 1992 39.2 -> 35.0
 // us, 512 x 1992 18.6 -> 10.4, 64 x 2999 26.0 -> 8.5, 1 x 2999 11.2 -> 6.2.
 template <bool SPLIT>
-__global__ void __launch_bounds__(256) fitness_kernel(const int* __restrict__ C, int ldc, int n,
+__global__ void fitness_kernel(const int* __restrict__ C, int ldc, int n,
                                const uint16_t* __restrict__ tours, int ldt, int count,
-                               long long* __restrict__ out, int log_split) {
+                               long long* __restrict__ out, int split) {
     __shared__ long long part[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, split = SPLIT ? 1 << log_split : 1;
-    const int w = (blockIdx.x * (blockDim.x >> 5) + warp) >> (SPLIT ? log_split : 0);
-    const int sub = SPLIT ? warp & (split - 1) : 0;
+    if (!SPLIT) split = 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w = (blockIdx.x * (blockDim.x >> 5) + warp) / split, sub = warp % split;
     long long f = 0;
     if (w < count) {
         const uint16_t* x = tours + (size_t)w * ldt;
@@ -637,7 +637,7 @@ int move_warps(const BatchView& b) {
 cudaError_t launch_fitness(const int* C, int ldc, int n, const uint16_t* tours, int ldt, int count,
                            long long* out, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    int log_split = 0;
+    int split = 1;
     // A tour of one round is not split, and eight of them share a block (4096
     // tours of 64: 5.5 us, in blocks of two 5.8); so do tours of two rounds, and
     // tours enough for eight blocks of eight per SM, where the number of blocks
@@ -651,14 +651,12 @@ cudaError_t launch_fitness(const int* C, int ldc, int n, const uint16_t* tours, 
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        while (log_split < 3 && (256 << log_split) < n &&
-               (2ll << log_split) * count <= 64 * sms)
-            ++log_split;
-        if (log_split > 0 || (n > 512 && count < 64 * sms)) threads = max(64, 32 << log_split);
+        while (split < 8 && 256 * split < n && 2ll * split * count <= 64 * sms) split *= 2;
+        if (split > 1 || (n > 512 && count < 64 * sms)) threads = max(64, 32 * split);
     }
-    const int per = threads / (32 << log_split);
-    auto* kern = log_split > 0 ? fitness_kernel<true> : fitness_kernel<false>;
-    kern<<<(count + per - 1) / per, threads, 0, st>>>(C, ldc, n, tours, ldt, count, out, log_split);
+    const int per = threads / (32 * split);
+    auto* kern = split > 1 ? fitness_kernel<true> : fitness_kernel<false>;
+    kern<<<(count + per - 1) / per, threads, 0, st>>>(C, ldc, n, tours, ldt, count, out, split);
     return cudaGetLastError();
 }
 
