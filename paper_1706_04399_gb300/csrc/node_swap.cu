@@ -52,7 +52,6 @@ using namespace tiled;
 constexpr unsigned long long kExact = 0x8000;
 constexpr unsigned long long kNone = ~0ull;
 constexpr int kNodeSwapMaxN = 4497;  // longer tours are refused (as the header says)
-constexpr int kThreadsPerSm = 640;  // the register budget's resident threads
 constexpr int kRowsStaged = 10;  // two swapped positions, two on each side
 
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
@@ -101,10 +100,12 @@ constexpr size_t swap_smem(int n, int warps, Costs costs) {
                (sizeof(unsigned long long) + 2 * sizeof(int) + 2 * sizeof(uint16_t));
 }
 
-// NT threads solve one tour; COLS: positions a thread holds in the first pass.
-template <int NT, Costs COSTS, int COLS>
-__global__ void __launch_bounds__(NT, COLS > 8 ? 3 : (NT == 96 ? 5 : kThreadsPerSm / NT))
-    node_swap_kernel(TwoOptBatch b) {
+// NT threads solve one tour; COLS: positions a thread holds in the first pass;
+// CTAS: blocks that an SM is to hold, which sets the registers of one (128
+// threads, 321 viewpoints, 127 tours: 2.43 ms with room for three blocks, 2.67
+// with room for five; 760 tours of 700 need the five).
+template <int NT, Costs COSTS, int COLS, int CTAS>
+__global__ void __launch_bounds__(NT, CTAS) node_swap_kernel(TwoOptBatch b) {
     constexpr int kW = NT / 32;
     constexpr bool kFull = COSTS == kMatrix, kRows = COSTS == kStaged;
     constexpr int kCols = COLS;
@@ -551,9 +552,9 @@ __global__ void __launch_bounds__(NT, COLS > 8 ? 3 : (NT == 96 ? 5 : kThreadsPer
     }
 }
 
-template <int NT, Costs COSTS, int COLS>
+template <int NT, Costs COSTS, int COLS, int CTAS>
 cudaError_t launch_nt(const TwoOptBatch& b, int num_sms, cudaStream_t st) {
-    auto* kern = node_swap_kernel<NT, COSTS, COLS>;
+    auto* kern = node_swap_kernel<NT, COSTS, COLS, CTAS>;
     const size_t smem = swap_smem(b.max_n, NT / 32, COSTS);
     cudaError_t e = raise_smem_limit(kern, smem);
     if (e != cudaSuccess) return e;
@@ -604,14 +605,16 @@ namespace {
 struct SwapConfig {
     int max_n, few, threads;
     Costs costs;
-    int cols;
+    int cols, ctas;
 };
 constexpr int kAny = INT_MAX;
 constexpr SwapConfig kConfigs[] = {
-    {64, kAny, 64, kMatrix, 2},     {100, kAny, 128, kMatrix, 2},   {160, 2, 128, kMatrix, 2},
-    {220, 1, 128, kMatrix, 2},      {1024, 2, 128, kStaged, 8},     {1500, 1, 256, kGlobal, 8},
-    {1500, 2, 128, kStaged, 12},    {768, 5, 96, kStaged, 8},       {600, kAny, 64, kStaged, 8},
-    {1024, kAny, 128, kStaged, 8},  {1500, kAny, 128, kStaged, 12}, {kNodeSwapMaxN, kAny, 256, kGlobal, 8},
+    {64, kAny, 64, kMatrix, 2, 10},     {100, kAny, 128, kMatrix, 2, 5},
+    {160, 2, 128, kMatrix, 2, 5},       {220, 1, 128, kMatrix, 2, 5},
+    {1024, 2, 128, kStaged, 8, 3},      {1500, 1, 256, kGlobal, 8, 2},
+    {1500, 2, 128, kStaged, 12, 3},     {768, 5, 96, kStaged, 8, 5},
+    {600, kAny, 64, kStaged, 8, 9},    {1024, kAny, 128, kStaged, 8, 5},
+    {1500, kAny, 128, kStaged, 12, 3},  {kNodeSwapMaxN, kAny, 256, kGlobal, 8, 2},
 };
 constexpr int kNumConfigs = sizeof(kConfigs) / sizeof(kConfigs[0]);
 
@@ -628,7 +631,7 @@ template <int K>
 cudaError_t launch_k(const TwoOptBatch& b, int k, int num_sms, cudaStream_t st) {
     constexpr SwapConfig c = kConfigs[K];
     static_assert(swap_smem(c.max_n, c.threads / 32, c.costs) <= 224 * 1024, "does not fit");
-    if (k == K) return launch_nt<c.threads, c.costs, c.cols>(b, num_sms, st);
+    if (k == K) return launch_nt<c.threads, c.costs, c.cols, c.ctas>(b, num_sms, st);
     if constexpr (K + 1 < kNumConfigs) return launch_k<K + 1>(b, k, num_sms, st);
     else return cudaErrorInvalidValue;
 }
