@@ -65,8 +65,8 @@
 // memory, so that one 8-byte gather brings both ends' costs to a city) and of
 // the new edges' pairs; for short ones the issue slots and the chain of a
 // pass, about 9000 cycles at n = 400.  Against scanning every row and every
-// pair of the new edges, on GB300: 600 tours at n = 1992 39 -> 28 ms, 150 at
-// n = 2999 28 -> 19, 600 at n = 1000 10.1 -> 7.1.
+// pair of the new edges, on GB300: 600 tours at n = 1992 39 -> 26 ms, 150 at
+// n = 2999 28 -> 18, 600 at n = 1000 10.1 -> 6.2.
 #include <climits>
 
 #include "tiled_common.cuh"
@@ -174,11 +174,12 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : kThreadsPerSm / NT))
     // are read in a few steps, are faster without (n = 400, 1024 tours: a swarm's
     // generations 8 % slower with them).
     constexpr bool kLists = ST == kCtaRows || ST == kGlobal;
-    // partners a thread has in flight (n = 400, 1024 tours, whole call: 1 3.39
-    // ms, 2 3.32, 4 3.73, 8 about 6: the rare path is unrolled with the common one)
+    // partners a thread has in flight (whole calls, one, two and four of them: 1024
+    // tours of 400 3.29, 3.27 and 3.34 ms, 150 of 2999 19.0, 18.0 and 18.2)
     constexpr int kBatch = 2;
     // threads per group of the choice of T' (see the head of the file): eight
-    // groups (16 groups 3.65 ms, 32 more)
+    // groups (four, eight and sixteen: 1024 tours of 400 3.22, 3.27 and 3.43 ms,
+    // 600 of 1000 6.42, 6.12 and 6.83)
     constexpr int kGroup = NT >= 256 ? 32 : (NT >= 128 ? 16 : 8);
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned long long s_key[2][kW];  // the warps' best, by pass parity
