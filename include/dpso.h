@@ -181,7 +181,8 @@ int dpso_two_opt(const int32_t *C_dev, int32_t n, uint16_t *tours_dev, int32_t c
  * array inside the library (held by every GPU that loads it, until exit) instead
  * of being allocated per call; it calls no allocating routine.  The kernel's
  * neighbour lists lie there too, or in one of the library's fixed scratch slots
- * (n <= 4096, and a slot is free), else it runs without them.
+ * (eight of 1 MiB, held likewise; n <= 4096, and a slot is free), else it runs
+ * without them.
  * For callers that must not allocate device memory while running: an on-board
  * re-planning loop whose GPU memory is reserved once at start-up (an
  * allocation can synchronise the device or fail under fragmentation in
